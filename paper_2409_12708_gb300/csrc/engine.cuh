@@ -73,14 +73,16 @@ struct Alloc {
 };
 
 // Stream-ordered scratch released in reverse order when it goes out of scope.
+// Every array starts on a 16-byte boundary whatever the caller's allocator
+// returns: the kernels read matrices in 16-byte chunks.
 struct Scratch {
     Alloc al;
     std::vector<void*> ptrs;
     explicit Scratch(const Alloc& a) : al(a) {}
     template <class X> X* get(size_t n) {
-        void* p = al.get(n * sizeof(X));
+        void* p = al.get(n * sizeof(X) + 15);
         ptrs.push_back(p);
-        return static_cast<X*>(p);
+        return reinterpret_cast<X*>((reinterpret_cast<uintptr_t>(p) + 15) & ~(uintptr_t)15);
     }
     void release() {
         for (auto it = ptrs.rbegin(); it != ptrs.rend(); ++it) al.put(*it);
@@ -211,13 +213,12 @@ struct Plan {
     int maxP = 0, maxN = 0;
 };
 
+// Launch shape (index into QR_SHAPES) of the QR of an m x n matrix.
 template <class T>
-inline void qr_params(int m, int n, int& nb) {
-    nb = sizeof(T) >= 8 ? 16 : 32;  // panel width (at most one warp of reflectors)
-    const size_t budget = 220 * 1024;
-    while (nb > 4 && qr_smem_bytes<T>(m, nb, n) > budget) nb /= 2;
-    if (qr_smem_bytes<T>(m, nb, n) > budget)
-        throw Error(THC_EUNSUPPORTED, "QR column length too large for shared memory");
+inline int qr_params(int m, int n, bool pivot) {
+    const int i = qr_shape<T>(m, n, pivot, 224 * 1024);
+    if (i < 0) throw Error(THC_EUNSUPPORTED, "QR column length too large for shared memory");
+    return i;
 }
 
 template <class T>
@@ -247,8 +248,7 @@ inline Plan make_plan(int mode, const std::vector<int>& inA, const std::vector<i
         P.maxL = std::max(P.maxL, (long)P.e[s] * P.k[s]);
         const int m = 4 * P.k[s + 1], n = P.e[s];
         if (s >= 1) {
-            int nb;
-            qr_params<T>(m, n, nb);
+            const int nb = QR_SHAPES[qr_params<T>(m, n, false)].nb;
             P.maxTw = std::max(P.maxTw, (long)ceil_div(std::min(m, n), nb) * nb * nb);
             P.maxQRm = std::max<long>(P.maxQRm, m);
         }
@@ -263,9 +263,7 @@ inline Plan make_plan(int mode, const std::vector<int>& inA, const std::vector<i
         P.maxP = std::max(P.maxP, p);
         P.maxN = std::max(P.maxN, n);
         if (m >= n) {
-            int nb;
-            qr_params<T>(m, n, nb);
-            P.maxTw = std::max(P.maxTw, (long)ceil_div(n, nb) * nb * nb);
+            qr_params<T>(m, n, true);  // refuses what no launch shape covers
             P.maxQRm = std::max<long>(P.maxQRm, m);
         }
     }

@@ -67,7 +67,10 @@ struct Engine {
     }
     static void set_attrs() {
         const int big = 1 << 30;
-        opt_in(k_qr<T>, big);
+        for (int i = 0; i < QR_NSHAPES; ++i) {
+            qr_dispatch<T, false>(i, [&](auto* k) { opt_in(k, big); });
+            qr_dispatch<T, true>(i, [&](auto* k) { opt_in(k, big); });
+        }
         opt_in(k_jacobi_select<T, 4>, big);
         opt_in(k_jacobi_select<T, 8>, big);
         opt_in(k_jacobi_select<T, 16>, big);
@@ -279,15 +282,14 @@ struct Engine {
                 job.strideT = w.sTw;
                 job.out = w.Lb[s & 1];
                 job.strideOut = w.sL;
-                qr_params<T>(job.m, job.n, job.nb);
+                const int shape = qr_params<T>(job.m, job.n, false);
                 if constexpr (std::is_same<T, float>::value)
-                    qt[s] = job.nb == QT_NB && job.m <= 1024 && (int)qt_smem_bytes(job.m) <= smem_optin - 2048;
+                    qt[s] = QR_SHAPES[shape].nb == QT_NB && job.m <= 1024 && (int)qt_smem_bytes(job.m) <= smem_optin - 2048;
                 job.mode = qt[s] ? QR_L_ONLY : QR_L_AND_Q;
                 job.colmap = nullptr;
-                job.pivot = 0;
                 {
                     THC_LAUNCH("qr_lq_sweep", st);
-                    k_qr<T><<<B, QR_THREADS, qr_smem_bytes<T>(job.m, job.nb, job.n), st>>>(job);
+                    launch_qr<false>(shape, job, B);
                 }
                 check();
             }
@@ -318,7 +320,6 @@ struct Engine {
                 colmap = w.perm;
                 QRJob<T> job;
                 job.colmap = w.perm;
-                job.pivot = 1;
                 job.A = w.W;
                 job.strideA = w.sC;
                 job.m = m;
@@ -328,11 +329,10 @@ struct Engine {
                 job.strideT = w.sTw;
                 job.out = w.Z;
                 job.strideOut = w.sZ;
-                qr_params<T>(m, n, job.nb);
                 job.mode = QR_R_ROWS;
                 {
                     THC_LAUNCH("qr_svd_precond", st);
-                    k_qr<T><<<B, QR_THREADS, qr_smem_bytes<T>(m, job.nb, n), st>>>(job);
+                    launch_qr<true>(qr_params<T>(m, n, true), job, B);
                 }
                 check();
             } else {
@@ -382,6 +382,13 @@ struct Engine {
                 gemm(B, P.out[s], 4 * P.k[s + 1], P.k[s], mop, qop, so);
             }
         }
+    }
+
+    template <bool PIV>
+    void launch_qr(int shape, const QRJob<T>& job, int B) {
+        const QrShape& sh = QR_SHAPES[shape];
+        const size_t smem = qr_smem_bytes<T>(sh, job.m, job.n, PIV);
+        qr_dispatch<T, PIV>(shape, [&](auto* k) { k<<<B, sh.threads(), smem, st>>>(job); });
     }
 
     // C = M_{s-1} Q_s from the reflectors the QR sweep left at site s (real

@@ -1,26 +1,44 @@
 // qr.cuh -- batched blocked Householder QR, one CTA per matrix.
 //
-// A (m x n, column-major, leading dimension ld, in global memory) is factored
-// as A = Q R with Q = H_0 H_1 ... H_{kk-1}, kk = min(m, n),
+// A (m x n, column-major, leading dimension ld, in global memory, m a multiple
+// of 4) is factored as A = Q R with Q = H_0 H_1 ... H_{kk-1}, kk = min(m, n),
 // H_j = I - tau_j v_j v_j^H, v_j(j) = 1, v_j(i < j) = 0 (Golub & Van Loan,
 // Householder QR; for complex A the reflector of LAPACK's convention, with a
 // real beta and a complex tau, and H_j^H applied to the trailing columns; the
 // blocked form uses the compact WY representation H_0 ... H_{b-1} =
-// I - V T V^H of Schreiber & Van Loan).  Panels of nb columns are factored in
-// shared memory; the trailing columns are updated in groups of QR_QG columns
-// straight from global memory with register-tiled products
-// (W = V^H Y, W <- T^H W, Y -= V W), so each group is read twice and written
-// once per panel.  Real and complex scalars share the code (scalar.cuh).
+// I - V T V^H of Schreiber & Van Loan).  Real and complex scalars share the
+// code (scalar.cuh).
+//
+// Work split.  Columns are held in registers, four ("a quad") per group of S
+// warps: lane l of warp h of the group holds 16-byte chunks of rows
+// ((q S + h) 32 + l) VEC, q < 4, of the four columns (64 registers).  The panel
+// of nb = 64 / S columns is factored by all groups at once, each on its own
+// quad; the finished reflectors V go to shared memory, and every trailing quad
+// then is loaded into registers once, updated (W = V^H Y, W <- T^H W,
+// Y -= V W) and stored once.  A group needs only its own warps for that (a
+// named barrier), so the groups run free of each other between panels and hide
+// one another's load latency; the CTA-wide barriers are one per panel column
+// (two when pivoting).  A 16-byte load of V from shared memory feeds four
+// columns, so the FMA pipe and the shared-memory pipe are about evenly loaded.
+// What bounds it: the panel columns' serial chain (norm, scalars, barrier, dots,
+// update: about 1500 cycles a column), then the FMA pipe of the updates (36 %
+// busy over the launch).  Measured (GB300, float32): 304 matrices of 1024 x 256
+// in 2.04 ms, one alone in 0.97 ms (4.55 and 2.14 ms with groups of 16 columns
+// updated straight from global memory behind four CTA barriers each); 304 of
+// 512 x 256 pivoted in 1.07 ms, one in 0.75 ms (3.43 and 1.69 ms).
 //
 // Modes (after the factorisation):
 //   QR_L_AND_Q : writes L = R^T (n x kk, row-major) and overwrites the first kk
 //                columns of A with the thin Q (used to right-canonicalise a site:
 //                A holds X^T, so X = L Q^T and Q^T becomes the site tensor; for
 //                complex X the plain transpose keeps Q^T's rows orthonormal).
-//   QR_R_ROWS  : writes R (n x n, row-major, zero below the diagonal); m >= n.
+//   QR_R_ROWS  : writes R (n x n, row-major, zero below the diagonal) of A with
+//                its columns reordered by block pivoting, and the order; m >= n.
 //   QR_L_ONLY  : writes L as QR_L_AND_Q and leaves the reflectors in A and the
 //                panel T matrices in Tw (Q is applied later without being formed).
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "scalar.cuh"
@@ -31,113 +49,85 @@ enum QRMode : int { QR_L_AND_Q = 1, QR_R_ROWS = 2, QR_L_ONLY = 3 };
 
 template <class T>
 struct QRJob {
-    T* A;          // term 0 matrix; term b at A + b * strideA
+    T* A;          // term 0 matrix; term b at A + b * strideA; columns 16-byte aligned
     long strideA;
     int m, n, ld;
     T* Tw;         // per-term panel T matrices, [ceil(kk/nb) * nb * nb]
     long strideT;
     T* out;        // L or R output
     long strideOut;
-    int nb;        // panel width
     int mode;
-    int* colmap;   // optional per-term column permutation (n ints, stride n):
-                   // logical column c is stored in physical column colmap[c]
-    int pivot;     // QR_R_ROWS only: choose the column order by block pivoting
-                   // (colmap is then an output: the chosen order)
+    int* colmap;   // QR_R_ROWS: output, the column order block pivoting chose (n ints, stride n)
 };
 
-// physical column of logical column c under the optional column map cm
-#define QCOL(c) (cm ? cm[(c)] : (c))
+constexpr int QR_NC = 4;  // columns of a quad
 
-constexpr int QR_THREADS = 512;  // 16 warps: one CTA per SM hides latency with more warps
-constexpr int QR_QG = 16;        // trailing columns per group
-
-// Column stride of the panel in shared memory: a multiple of 16 bytes (vector
-// access to 4 consecutive rows) that is 16 bytes past a multiple of 128, so
-// the columns a warp reads at once fall in distinct bank groups.
 template <class T>
-__host__ __device__ inline int qr_ldp(int m) {
-    constexpr int e16 = 16 / (int)sizeof(T), e128 = 128 / (int)sizeof(T);
-    return (m + e128 - 1) / e128 * e128 + e16;
+struct QrVec {  // rows per 16-byte chunk
+    static constexpr int V = 16 / (int)sizeof(T);
+};
+
+// A launch shape: panels of NB columns, S warps per quad, NQ chunks per lane and
+// column.  It covers 32 VEC S NQ rows with 32 S NB / 4 threads.
+struct QrShape {
+    int nb, s, nq;
+    int threads() const { return 32 * s * nb / QR_NC; }
+    int units() const { return s * nq; }  // rows covered, in 32 VEC
+};
+// The first that covers the matrix is taken.  One warp per quad needs no barrier
+// between the warps of a quad, and two CTAs fit on an SM, so that one's panel (a
+// serial chain) overlaps the other's update: 304 pivoted 512 x 256 float32
+// matrices take 1.07 ms that way and 1.57 ms with two warps per quad, and one
+// matrix alone 0.75 against 0.77 ms.
+constexpr QrShape QR_SHAPES[] = {{32, 1, 2}, {32, 1, 4}, {32, 2, 4}, {16, 4, 4}, {8, 8, 4}, {4, 16, 4}};
+constexpr int QR_NSHAPES = 6;
+
+// Chunks per lane and column that a panel of R rows works on: all or half of
+// them, so that the inner loops have no branch per chunk.
+__host__ __device__ inline int qr_active(int R, int vec, int s, int nq) {
+    return R > 32 * vec * s * (nq / 2) ? nq : nq / 2;
+}
+// Column stride of V in shared memory: the rows those chunks cover.
+template <class T>
+__host__ __device__ inline int qr_ldp(int m, int s, int nq) {
+    return 32 * QrVec<T>::V * s * qr_active(m, QrVec<T>::V, s, nq);
 }
 
-// Reflector rows per lane in the register-tiled products (lane (ig, cg) owns
-// rows ig + 8 ii of W, ii < qr_ni(nb), and columns 4 cg .. 4 cg + 3).
-__host__ __device__ inline int qr_ni(int nb) { return nb >= 32 ? 4 : (nb >= 16 ? 2 : 1); }
-
+// Shared memory: norm partials and alphas (16 bytes a warp), V, panel dots, the
+// groups' W and W partials, T and G = V^H V; then the pivoting state.
 template <class T>
-__host__ inline size_t qr_smem_bytes(int m, int nb, int n) {
-    const size_t cap = 8 * qr_ni(nb);  // rows of W per warp partial
-    const size_t base = 64 * sizeof(double) + (size_t)nb * qr_ldp<T>(m) * sizeof(T) + 2 * (size_t)nb * nb * sizeof(T) +
-                        ((size_t)(QR_THREADS / 32) * cap * QR_QG + 2 * cap * QR_QG) * sizeof(T);
-    // pivoting state: nb float64 norms, nb + n (real) metrics / norms, two n-int column maps
-    const size_t piv = (size_t)nb * sizeof(double) + (size_t)(nb + n) * sizeof(real_t<T>) +
-                       2 * (size_t)n * sizeof(int);
-    return base + ((piv + 15) & ~(size_t)15);
+__host__ inline size_t qr_smem_bytes(const QrShape& sh, int m, int n, bool pivot) {
+    const size_t nb = sh.nb, warps = sh.threads() / 32;
+    const size_t elems = nb * qr_ldp<T>(m, sh.s, sh.nq) + 2 * warps * QR_NC + (nb / QR_NC) * (sh.s + 1) * QR_NC * nb + 2 * nb * (nb + 4);
+    const size_t piv = pivot ? (nb + n) * sizeof(real_t<T>) + 2 * (size_t)n * sizeof(int) : 0;
+    return elems * sizeof(T) + 3 * warps * 16 + ((piv + 15) & ~(size_t)15);
 }
 
-// four consecutive elements with 16-byte accesses (p 16-byte aligned)
+// The shape for m rows (negative: none).
 template <class T>
-__device__ __forceinline__ void ld4(T (&x)[4], const T* p) {
-    if constexpr (is_complex_v<T>) {
-        constexpr int NV = 4 * (int)sizeof(T) / 16;  // 16-byte words
-        uint4 u[NV];
-#pragma unroll
-        for (int q = 0; q < NV; ++q) u[q] = reinterpret_cast<const uint4*>(p)[q];
-        const T* pu = reinterpret_cast<const T*>(u);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = pu[q];
-    } else if constexpr (sizeof(T) == 4) {
-        const float4 u = *reinterpret_cast<const float4*>(p);
-        x[0] = u.x;
-        x[1] = u.y;
-        x[2] = u.z;
-        x[3] = u.w;
-    } else {
-        const double2 a = *reinterpret_cast<const double2*>(p);
-        const double2 b = *reinterpret_cast<const double2*>(p + 2);
-        x[0] = a.x;
-        x[1] = a.y;
-        x[2] = b.x;
-        x[3] = b.y;
+__host__ inline int qr_shape(int m, int n, bool pivot, size_t smem_max) {
+    for (int i = 0; i < QR_NSHAPES; ++i) {
+        if (QR_SHAPES[i].units() * 32 * QrVec<T>::V < m) continue;
+        if (qr_smem_bytes<T>(QR_SHAPES[i], m, n, pivot) <= smem_max) return i;
     }
+    return -1;
+}
+
+// 16-byte chunk load / store
+template <class T>
+__device__ __forceinline__ void qr_ld(T (&x)[QrVec<T>::V], const T* p) {
+    const uint4 u = *reinterpret_cast<const uint4*>(p);
+    const T* pu = reinterpret_cast<const T*>(&u);
+#pragma unroll
+    for (int e = 0; e < QrVec<T>::V; ++e) x[e] = pu[e];
 }
 template <class T>
-__device__ __forceinline__ void st4(T* p, const T (&x)[4]) {
-    if constexpr (is_complex_v<T>) {
-        constexpr int NV = 4 * (int)sizeof(T) / 16;
-        uint4 u[NV];
-        T* pu = reinterpret_cast<T*>(u);
+__device__ __forceinline__ void qr_st(T* p, const T (&x)[QrVec<T>::V]) {
+    uint4 u;
+    T* pu = reinterpret_cast<T*>(&u);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) pu[q] = x[q];
-#pragma unroll
-        for (int q = 0; q < NV; ++q) reinterpret_cast<uint4*>(p)[q] = u[q];
-    } else if constexpr (sizeof(T) == 4) {
-        *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-    } else {
-        *reinterpret_cast<double2*>(p) = make_double2(x[0], x[1]);
-        *reinterpret_cast<double2*>(p + 2) = make_double2(x[2], x[3]);
-    }
-}
-// rows r .. r+3 of a global column (zeros at or beyond R); vector access when allowed
-template <class T>
-__device__ __forceinline__ void ld4_col(T (&x)[4], const T* col, int r, int R, bool vec) {
-    if (vec && r + 4 <= R) {
-        ld4(x, col + r);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = r + q < R ? col[r + q] : tzero<T>();
-    }
-}
-template <class T>
-__device__ __forceinline__ void st4_col(T* col, const T (&x)[4], int r, int R, bool vec) {
-    if (vec && r + 4 <= R) {
-        st4(col + r, x);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (r + q < R) col[r + q] = x[q];
-    }
+    for (int e = 0; e < QrVec<T>::V; ++e) pu[e] = x[e];
+    *reinterpret_cast<uint4*>(p) = u;
 }
 
 // Squared norm with about twice the storage precision.  A Householder
@@ -152,6 +142,7 @@ template <>
 struct SqAcc<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double x) { s += x * x; }
+    __device__ __forceinline__ void merge(const SqAcc& o) { s += o.s; }
     __device__ __forceinline__ double warp_total() { return warp_sum(s); }
 };
 template <>
@@ -163,17 +154,20 @@ struct SqAcc<float> {
         lo += ((hi - (s - bp)) + (p - bp)) + e;
         hi = s;
     }
+    __device__ __forceinline__ void merge(const SqAcc& o) {
+        const float s = hi + o.hi, bp = s - hi;
+        lo = (lo + o.lo) + ((hi - (s - bp)) + (o.hi - bp));
+        hi = s;
+    }
     // butterfly of float-float pairs; every lane ends with the same total
-    __device__ __forceinline__ double warp_total() {
+    __device__ __forceinline__ void warp_fold() {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-            const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-            const float s = hi + h2, bp = s - hi;
-            lo = (lo + l2) + ((hi - (s - bp)) + (h2 - bp));
-            hi = s;
+            SqAcc b;
+            b.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+            b.lo = __shfl_xor_sync(0xffffffffu, lo, o);
+            merge(b);
         }
-        return (double)hi + (double)lo;
     }
 };
 
@@ -185,8 +179,10 @@ struct SqAcc<cplx<R>> {
         a.add(x.x);
         a.add(x.y);
     }
-    __device__ __forceinline__ double warp_total() { return a.warp_total(); }
+    __device__ __forceinline__ void merge(const SqAcc& o) { a.merge(o.a); }
 };
+
+
 
 // |x|^2 evaluated in float64
 template <class T>
@@ -195,544 +191,767 @@ __device__ __forceinline__ double dabs2(T x) {
     else return (double)x * (double)x;
 }
 
-// Squared norm of y[r0 .. R) by one warp (every lane gets the total).  In
-// float32, squares of entries below ~1e-19 underflow or lose their precision
-// (residues of rank-deficient columns are of that size), which would make the
-// reflector inconsistent with its vector; such small totals are recomputed
-// from float64 squares.
+// acc += sum_e conj(v_e) y_e over one chunk, y -= v w over one chunk.  float32
+// runs on packed pairs (two IEEE FMAs per instruction).
 template <class T>
-__device__ __forceinline__ double col_norm2(const T* y, int r0, int R) {
-    const int lane = threadIdx.x & 31;
-    SqAcc<T> a;
-    for (int r = r0 + lane; r < R; r += 32) a.add(y[r]);
-    double t = a.warp_total();
-    if (sizeof(real_t<T>) == 4 && t < 1e-30) {
-        double s = 0.0;
-        for (int r = r0 + lane; r < R; r += 32) s += dabs2(y[r]);
-        t = warp_sum(s);
+struct QrAcc {
+    T a = tzero<T>();
+    __device__ __forceinline__ void add(const T (&v)[QrVec<T>::V], const T (&y)[QrVec<T>::V]) {
+#pragma unroll
+        for (int e = 0; e < QrVec<T>::V; ++e) a += tconj_mul(v[e], y[e]);
     }
+    __device__ __forceinline__ T total() const { return a; }
+};
+template <>
+struct QrAcc<float> {
+    float2 a = {0.f, 0.f};
+    __device__ __forceinline__ void add(const float (&v)[4], const float (&y)[4]) {
+        a = __ffma2_rn(make_float2(v[0], v[1]), make_float2(y[0], y[1]), a);
+        a = __ffma2_rn(make_float2(v[2], v[3]), make_float2(y[2], y[3]), a);
+    }
+    __device__ __forceinline__ float total() const { return a.x + a.y; }
+};
+template <class T>
+__device__ __forceinline__ void qr_axpy(T (&y)[QrVec<T>::V], const T (&v)[QrVec<T>::V], T nw) {  // y += v nw
+    if constexpr (std::is_same<T, float>::value) {
+        const float2 w2 = make_float2(nw, nw);
+        const float2 a = __ffma2_rn(make_float2(v[0], v[1]), w2, make_float2(y[0], y[1]));
+        const float2 b = __ffma2_rn(make_float2(v[2], v[3]), w2, make_float2(y[2], y[3]));
+        y[0] = a.x;
+        y[1] = a.y;
+        y[2] = b.x;
+        y[3] = b.y;
+    } else {
+#pragma unroll
+        for (int e = 0; e < QrVec<T>::V; ++e) y[e] += v[e] * nw;
+    }
+}
+
+// Reduce-scatter of NV per-lane values over the warp: the lanes of group i
+// (lane / (32 / NV)) return value i's total.
+template <int NV, class T>
+__device__ __forceinline__ T qr_reduce_scatter(T (&v)[NV]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int lev = 0; (1 << lev) < NV; ++lev) {
+        const int o = 16 >> lev, half = (NV >> lev) / 2;
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < NV / 2; ++i) {
+            if (i < half) {
+                const T send = upper ? v[i] : v[half + i];
+                const T keep = upper ? v[half + i] : v[i];
+                v[i] = keep + shfl_xor(send, o);
+            }
+        }
+    }
+    T t = v[0];
+#pragma unroll
+    for (int o = 32 / NV / 2; o >= 1; o >>= 1) t += shfl_xor(t, o);
     return t;
 }
 
-// Register-tiled pieces of the compact-WY update with the panel's V held
-// explicitly in shared memory (column i at P + i*ldp: zeros above row i, 1 at
-// row i, zero rows from R up to the next multiple of 4).
-//
-// (1) Per-warp partial products Wp[w] = V^H Y over the rows of warp w for the
-//     QR_QG columns whose bases col(c) returns (c < QR_QG; null: no column).
-//     Lane (ig, cg) owns rows ig + 8 ii of W and columns 4 cg .. 4 cg + 3; each
-//     step takes four rows of V and Y with 16-byte loads.
-template <class T, int NI, class ColF>
-__device__ __forceinline__ void qr_vty(const T* P, int ldp, int pw, int R, T* Wp, ColF col, bool vec) {
-    constexpr int CAP = 8 * NI;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int ig = lane >> 2, cg = lane & 3;
-    const int R4 = ceil_div(R, 4), qpw = ceil_div(R4, nw);
-    const int r0 = 4 * wid * qpw, r1 = min(R, 4 * (wid + 1) * qpw);
-    T acc[NI][4];
+// A warp's squared norm (float-float or float64), passed through shared memory
+// and folded over the warps of a group.
+template <class RT>
+struct QrNorm;
+template <>
+struct QrNorm<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void of(SqAcc<double> a) { s = warp_sum(a.s); }
+    __device__ __forceinline__ void store(unsigned char* p) const { *reinterpret_cast<double*>(p) = s; }
+    __device__ __forceinline__ void fold(const unsigned char* p) { s += *reinterpret_cast<const double*>(p); }
+    __device__ __forceinline__ double value() const { return s; }
+    __device__ __forceinline__ double wide() const { return s; }
+};
+template <>
+struct QrNorm<float> {
+    SqAcc<float> a;
+    __device__ __forceinline__ void of(SqAcc<float> b) {
+        b.warp_fold();
+        a = b;
+    }
+    __device__ __forceinline__ void store(unsigned char* p) const {
+        *reinterpret_cast<float2*>(p) = make_float2(a.hi, a.lo);
+    }
+    __device__ __forceinline__ void fold(const unsigned char* p) {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        SqAcc<float> b;
+        b.hi = t.x;
+        b.lo = t.y;
+        a.merge(b);
+    }
+    __device__ __forceinline__ float value() const { return a.hi + a.lo; }
+    __device__ __forceinline__ double wide() const { return (double)a.hi + (double)a.lo; }
+    __device__ __forceinline__ float plus_square(float x) const {
+        SqAcc<float> b = a;
+        b.add(x);
+        return b.hi + b.lo;
+    }
+};
+template <class T>
+__device__ __forceinline__ SqAcc<T> qr_real_acc(const SqAcc<T>& a) { return a; }
+template <class R>
+__device__ __forceinline__ SqAcc<R> qr_real_acc(const SqAcc<cplx<R>>& a) { return a.a; }
+
+// sqrt(a2), (|x| + sqrt(a2)) / sqrt(a2) and 1 / (|x| + sqrt(a2)) for the reflector, from the
+// hardware's float32 reciprocal (square root) and Newton / Halley steps: one
+// short dependent chain instead of a square root and two divisions, each right
+// to about an ulp.  float64: a2 in float32's range.
+__device__ __forceinline__ void qr_scalars(float a2, float ax, float& nrm, float& quo, float& inv) {
+    float r = rsqrtf(a2);
+    r = fmaf(0.5f * r, fmaf(-(a2 * r), r, 1.f), r);
+    nrm = a2 * r;
+    nrm = fmaf(0.5f * r, fmaf(-nrm, nrm, a2), nrm);
+    const float d = ax + nrm;
+    quo = d * r;
+    quo = fmaf(r, fmaf(-quo, nrm, d), quo);
+    inv = __fdividef(1.f, d);
+    inv = fmaf(inv, fmaf(-d, inv, 1.f), inv);
+}
+__device__ __forceinline__ double qr_recip(double d) {
+    const double r = (double)__fdividef(1.f, (float)d);
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double qr_root(double a2, double& r) {  // sqrt(a2) and r = 1 / sqrt(a2)
+    r = (double)rsqrtf((float)a2);
+    const double e = fma(-(a2 * r), r, 1.0);
+    r = fma(r * e, fma(0.375, e, 0.5), r);
+    const double n = a2 * r;
+    return fma(0.5 * r, fma(-n, n, a2), n);
+}
+__device__ __forceinline__ void qr_scalars(double a2, double ax, double& nrm, double& quo, double& inv) {
+    double r;
+    nrm = qr_root(a2, r);
+    const double d = ax + nrm;
+    quo = d * r;
+    quo = fma(r, fma(-quo, nrm, d), quo);
+    inv = qr_recip(d);
+}
+// the exponents of a sum of squares and of its part leave room for the above
+__device__ __forceinline__ bool qr_in_range(double part, double a2) {  // 2^-100 < part, a2 < 2^100
+    return __double2hiint(part) > 923 << 20 && __double2hiint(a2) < 1123 << 20;
+}
+
+// What a warp knows of its place, and the CTA's shared arrays.
+template <class T, int NB, int S, int NQ>
+struct QrCtx {
+    static constexpr int V = QrVec<T>::V;
+    static constexpr int NG = NB / QR_NC;        // groups
+    static constexpr int WARPS = NG * S;
+    static constexpr int LDT = NB + 1;           // leading dimension of T and G
+    static constexpr int GSZ = (S + 1) * QR_NC * NB;
+    int ldp, grp, h, lane;
+    T *P, *Tm, *G;  // V (column i at P + i ldp), T and G
+    T *Wp, *W1;     // this group's W partials [h][c][i] and W [i][4]
+    T* pd;          // panel dots [parity][warp][4]
+    unsigned char *pn, *pa;  // norm partials [parity][warp], alpha [group] (16 bytes each)
+    __device__ __forceinline__ int row(int q) const { return ((q * S + h) * 32 + lane) * V; }
+    __device__ __forceinline__ void sync() const {  // the group's warps
+        if constexpr (S == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(32 * S) : "memory");
+    }
+};
+
+// Four columns in registers.
+template <class T, int NQ>
+using QrQuad = T[QR_NC][NQ][QrVec<T>::V];
+
+template <class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_load(const QrCtx<T, NB, S, NQ>& x, QrQuad<T, NQ>& y, T* const (&col)[QR_NC], int R) {
 #pragma unroll
-    for (int ii = 0; ii < NI; ++ii)
+    for (int q = 0; q < NQ; ++q) {
+        const int r = x.row(q);
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) acc[ii][jj] = tzero<T>();
-    const T* yc[4];
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) yc[jj] = col(4 * cg + jj);
-    for (int r = r0; r < r1; r += 4) {
-        T v[NI][4], y[4][4];
-#pragma unroll
-        for (int ii = 0; ii < NI; ++ii) {
-            if (ig + 8 * ii < pw) {
-                ld4(v[ii], P + (ig + 8 * ii) * ldp + r);
+        for (int c = 0; c < QR_NC; ++c) {
+            if (r < R && col[c]) {
+                qr_ld(y[c][q], col[c] + r);
             } else {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) v[ii][q] = tzero<T>();
+                for (int e = 0; e < QrVec<T>::V; ++e) y[c][q][e] = tzero<T>();
             }
         }
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            if (yc[jj]) {
-                ld4_col(y[jj], yc[jj], r, R, vec);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) y[jj][q] = tzero<T>();
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int ii = 0; ii < NI; ++ii)
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += tconj_mul(v[ii][q], y[jj][q]);
-    }
-#pragma unroll
-    for (int ii = 0; ii < NI; ++ii)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) Wp[(wid * CAP + ig + 8 * ii) * QR_QG + 4 * cg + jj] = acc[ii][jj];
-}
-
-// (2) W0 = sum of the warp partials (pw x QR_QG)
-template <class T>
-__device__ __forceinline__ void qr_sum_partials(const T* Wp, T* W0, int pw, int cap) {
-    const int nw = blockDim.x >> 5;
-    for (int o = threadIdx.x; o < pw * QR_QG; o += blockDim.x) {
-        T s = tzero<T>();
-        for (int w = 0; w < nw; ++w) s += Wp[w * cap * QR_QG + o];
-        W0[o] = s;
     }
 }
-
-// (3) W1 = T^H W0 (factorisation) or T W0 (forming Q); T upper triangular
-template <class T>
-__device__ __forceinline__ void qr_t_times(const T* Tm, int nbT, const T* W0, T* W1, int pw, bool transpose) {
-    for (int o = threadIdx.x; o < pw * QR_QG; o += blockDim.x) {
-        const int i = o / QR_QG, c = o % QR_QG;
-        T s = tzero<T>();
-        if (transpose) {
-            for (int l = 0; l <= i; ++l) s += tconj_mul(Tm[l * nbT + i], W0[l * QR_QG + c]);
-        } else {
-            for (int l = i; l < pw; ++l) s += Tm[i * nbT + l] * W0[l * QR_QG + c];
-        }
-        W1[o] = s;
-    }
-}
-
-// (4) Y -= V W1 for ncols (<= QR_QG) columns, each thread a tile of 4 rows x 4
-//     columns (consecutive threads: consecutive row quads of a column quad).
-//     col(c) gives the base of column c in global memory.  IDENT: Y starts as
-//     the identity columns (local row cb + c of column c is 1) instead of
-//     being loaded.
-template <class T, bool IDENT, class ColF>
-__device__ __forceinline__ void qr_sub_vw(const T* P, int ldp, int pw, int R, const T* W1, int ncols, int cb,
-                                          ColF col, bool vec) {
-    const int R4 = ceil_div(R, 4), ncq = ceil_div(ncols, 4);
-    for (int t = threadIdx.x; t < R4 * ncq; t += blockDim.x) {
-        const int cq = t / R4, r = 4 * (t - cq * R4);
-        T* yc[4];
-        T y[4][4];
+template <class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_store(const QrCtx<T, NB, S, NQ>& x, const QrQuad<T, NQ>& y, T* const (&col)[QR_NC], int R) {
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const int c = 4 * cq + jj;
-            yc[jj] = c < ncols ? col(c) : nullptr;
-            if (IDENT) {
+    for (int q = 0; q < NQ; ++q) {
+        const int r = x.row(q);
+        if (r < R) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) y[jj][q] = (r + q == cb + c) ? tone<T>() : tzero<T>();
-            } else if (yc[jj]) {
-                ld4_col(y[jj], yc[jj], r, R, vec);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) y[jj][q] = tzero<T>();
-            }
-        }
-        T acc[4][4];
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[jj][q] = tzero<T>();
-#pragma unroll 4
-        for (int i = 0; i < pw; ++i) {
-            T vq[4], w[4];
-            ld4(vq, P + i * ldp + r);
-            ld4(w, W1 + i * QR_QG + 4 * cq);
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[jj][q] += vq[q] * w[jj];
-        }
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) y[jj][q] -= acc[jj][q];
-            if (yc[jj]) st4_col(yc[jj], y[jj], r, R, vec);
+            for (int c = 0; c < QR_NC; ++c)
+                if (col[c]) qr_st(col[c] + r, y[c][q]);
         }
     }
 }
 
-// Apply (H_p0 ... H_{p0+pw-1})^H (transpose=true, factorisation) or
-// H_p0 ... H_{p0+pw-1} (transpose=false, forming Q) to columns [c_begin, c_end)
-// of A, rows [p0, m), in groups of QR_QG columns: W = V^H Y, W <- T^H W (or
-// T W), Y -= V W.  Every product step is 16-byte loads and an outer product
-// of 4-vectors.
-template <class T, int NI>
-__device__ void qr_block_apply(T* A, int ld, int m, int p0, int pw, int c_begin, int c_end, const T* P, int ldp,
-                               const T* Tm, int nbT, T* Wp, T* W0, T* W1, bool transpose, const int* cm,
-                               bool vec) {
-    const int R = m - p0;
-    for (int c0 = c_begin; c0 < c_end; c0 += QR_QG) {
-        auto col = [&](int c) -> T* {
-            const int cc = c0 + c;
-            return cc < c_end ? A + (long)QCOL(cc) * ld + p0 : nullptr;
-        };
-        qr_vty<T, NI>(P, ldp, pw, R, Wp, col, vec);
-        __syncthreads();
-        qr_sum_partials(Wp, W0, pw, 8 * NI);
-        __syncthreads();
-        qr_t_times(Tm, nbT, W0, W1, pw, transpose);
-        __syncthreads();
-        qr_sub_vw<T, false>(P, ldp, pw, R, W1, min(QR_QG, c_end - c0), 0, col, vec);
-        __syncthreads();
-    }
-}
-
-// Columns p0 .. p0+pw-1 of Q = H_0 ... H_{kk-1} [I; 0] once the later panels
-// are applied: rows p0.. of those columns are H_p0 ... H_{p0+pw-1} E with E the
-// identity columns, i.e. E - V (T V1^H) with V1 the top pw x pw block of V
-// (V^H E = V1^H); rows above p0 are zero.
-template <class T>
-__device__ void qr_form_panel(T* A, int ld, int m, int p0, int pw, const T* P, int ldp, const T* Tm, int nbT,
-                              T* W0, T* W1, const int* cm, bool vec) {
-    const int R = m - p0;
-    for (int cb = 0; cb < pw; cb += QR_QG) {
-        const int gc = min(QR_QG, pw - cb);
-        for (int o = threadIdx.x; o < pw * QR_QG; o += blockDim.x) {
-            const int i = o / QR_QG, c = o % QR_QG;
-            W0[o] = c < gc ? tconj(P[i * ldp + cb + c]) : tzero<T>();
+// Y <- (I - V T^H V^H) Y (adj: the factorisation) or (I - V T V^H) Y (forming
+// Q) on a quad, by one group; NA chunks are worked on.
+template <int NA, class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_apply_quad(const QrCtx<T, NB, S, NQ>& x, QrQuad<T, NQ>& y, int pw, bool adj) {
+    constexpr int V = QrVec<T>::V, IB = 2;
+    const T* vrow = x.P + x.row(0);
+#pragma unroll 1
+    for (int i0 = 0; i0 < pw; i0 += IB) {  // W = V^H Y (column pw of V, read when pw is odd, is discarded)
+        QrAcc<T> acc[IB * QR_NC];
+#pragma unroll
+        for (int ii = 0; ii < IB; ++ii) {
+            T v[NA][V];
+#pragma unroll
+            for (int q = 0; q < NA; ++q) qr_ld(v[q], vrow + (i0 + ii) * x.ldp + q * 32 * V * S);
+#pragma unroll
+            for (int q = 0; q < NA; ++q)
+#pragma unroll
+                for (int c = 0; c < QR_NC; ++c) acc[ii * QR_NC + c].add(v[q], y[c][q]);
         }
-        __syncthreads();
-        qr_t_times(Tm, nbT, W0, W1, pw, false);
-        __syncthreads();
-        auto col = [&](int c) -> T* { return A + (long)QCOL(p0 + cb + c) * ld + p0; };
-        qr_sub_vw<T, true>(P, ldp, pw, R, W1, gc, cb, col, vec);
-        __syncthreads();
+        T w[IB * QR_NC];
+#pragma unroll
+        for (int k = 0; k < IB * QR_NC; ++k) w[k] = acc[k].total();
+        const T t = qr_reduce_scatter<IB * QR_NC>(w);
+        constexpr int GL = 32 / (IB * QR_NC);  // lanes per value
+        const int k = x.lane / GL;
+        if (x.lane % GL == 0) x.Wp[(x.h * QR_NC + k % QR_NC) * NB + i0 + k / QR_NC] = t;
     }
-    for (int i = threadIdx.x; i < pw * p0; i += blockDim.x) {
-        const int c = i / p0, r = i % p0;
-        A[(long)QCOL(p0 + c) * ld + r] = tzero<T>();
+    x.sync();
+#pragma unroll 1
+    for (int c = x.h; c < QR_NC; c += S) {  // W <- T^H W (T W): lane i forms row i
+        const int i = x.lane;
+        T w0 = tzero<T>(), w1 = tzero<T>();
+        if (i < pw)
+#pragma unroll
+            for (int hh = 0; hh < S; ++hh) w0 += x.Wp[(hh * QR_NC + c) * NB + i];
+        const T* t = adj ? x.Tm + (i < NB ? i : 0) : x.Tm + (i < NB ? i : 0) * x.LDT;
+        const int st = adj ? x.LDT : 1;
+#pragma unroll 8
+        for (int l = 0; l < pw; ++l) {
+            const T tl = t[l * st];
+            w1 += (adj ? tconj(tl) : tl) * shfl(w0, l);
+        }
+        if (i < pw) x.W1[i * QR_NC + c] = tzero<T>() - w1;
     }
-    __syncthreads();
+    x.sync();
+#pragma unroll 2
+    for (int i = 0; i < pw; ++i) {  // Y -= V W
+        T w[QR_NC], v[NA][V];
+#pragma unroll
+        for (int q = 0; q < NA; ++q) qr_ld(v[q], vrow + i * x.ldp + q * 32 * V * S);
+#pragma unroll
+        for (int c = 0; c < QR_NC; c += V) {
+            T t[V];
+            qr_ld(t, x.W1 + i * QR_NC + c);
+#pragma unroll
+            for (int e = 0; e < V; ++e) w[c + e] = t[e];
+        }
+#pragma unroll
+        for (int q = 0; q < NA; ++q)
+#pragma unroll
+            for (int c = 0; c < QR_NC; ++c) qr_axpy(y[c][q], v[q], w[c]);
+    }
 }
 
-// Panel in shared memory as explicit V: zeros above the diagonal, 1 on it.
-template <class T>
-__device__ __forceinline__ void qr_explicit_v(T* P, int ldp, int pw) {
-    for (int o = threadIdx.x; o < pw * pw; o += blockDim.x) {
-        const int i = o / pw, r = o % pw;  // column i, row r
-        if (r <= i) P[i * ldp + r] = (r == i) ? tone<T>() : tzero<T>();
-    }
-}
-
-// Unblocked Householder factorisation of the panel P (R rows, zero-padded)
-// with two barriers per column: thread 0 forms reflector j from alpha = P[j][j]
-// and the squared norm below it (computed by the warp that updated the column
-// in the previous step); then every warp applies H_j to its panel columns with
-// the unscaled x (the scale 1/(alpha - beta) is applied inside the dot and the
-// update), forms the next norm(s), and all threads scale the previous column,
-// which no longer is read.  tau_j goes to Tm[j][j], beta_j to P[j][j].
-// Pivoting (pmp != null, the panel's slice of the column map): before step j
-// thread 0 picks the remaining column with the largest norm below row j-1
-// (alpha^2 + ||x||^2), the columns are swapped in P and in pmp (a third
-// barrier), and every warp keeps the norms of all its columns current.
-template <class T>
-__device__ void qr_panel(T* P, int ldp, int R, int pw, T* Tm, int nb, T* psc, double* red, int* pmp, double* nb2,
-                         real_t<T>* met) {
+// Reflector of a column (y, held by the owner group), step j of the panel: its
+// squared norm below row j in about twice the storage precision, beta, tau and
+// the scaled v, which goes to V's column j (zeros above row j, 1 on it).  The
+// registers keep R's rows above j, beta on row j and v below.
+template <int NA, class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_reflect(const QrCtx<T, NB, S, NQ>& x, T (&y)[NQ][QrVec<T>::V], int j) {
+    constexpr int V = QrVec<T>::V;
     using RT = real_t<T>;
-    __shared__ int ksh;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-    const bool piv = pmp != nullptr;
-    const int R4 = 4 * ceil_div(R, 4);
-    if (!piv) {
-        if (wid == 0) {
-            const double t = col_norm2(P, 1, R);
-            if (lane == 0) red[0] = t;
-        }
-    } else {
-        for (int c = wid; c < pw; c += nw) {
-            const double t = col_norm2(P + c * ldp, 1, R);
-            if (lane == 0) {
-                nb2[c] = t;
-                met[c] = RT(dabs2(P[c * ldp]) + t);
+    SqAcc<T> a[NA];
+#pragma unroll
+    for (int e = 0; e < V; ++e)
+#pragma unroll
+        for (int q = 0; q < NA; ++q) a[q].add(x.row(q) + e > j ? y[q][e] : tzero<T>());
+#pragma unroll
+    for (int q = 1; q < NA; ++q) a[0].merge(a[q]);
+    const int par = j & 1;
+    unsigned char* pn = x.pn + (size_t)(par * x.WARPS + x.grp * S) * 16;
+    T* alpha_sh = reinterpret_cast<T*>(x.pa + (size_t)x.grp * 16);
+    QrNorm<RT> nrm;
+    nrm.of(qr_real_acc(a[0]));
+    if (S > 1 && x.lane == 0) nrm.store(pn + x.h * 16);
+    if (x.h == 0) {  // row j < 32 VEC lies in the first chunk of warp 0
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+            if (x.row(0) + e == j) *alpha_sh = y[0][e];
+    }
+    x.sync();
+    if constexpr (S > 1) {
+        nrm = QrNorm<RT>{};
+#pragma unroll 1
+        for (int hh = 0; hh < S; ++hh) nrm.fold(pn + hh * 16);
+    }
+    const T alpha = *alpha_sh;
+    double xn2 = 0.0;
+    bool tiny = false;
+    if constexpr (sizeof(RT) == 4) tiny = nrm.value() < 1e-30f;
+    if (tiny) {
+        // squares of entries below ~1e-19 (residues of rank-deficient columns)
+        // underflow in float32: such totals are recomputed from float64 squares
+        double s = 0.0;
+#pragma unroll 1
+        for (int r = x.row(0), q = 0; q < NA; ++q, r += 32 * V * S)
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                T t = y[0][e];
+#pragma unroll
+                for (int k = 1; k < NA; ++k) t = q == k ? y[k][e] : t;
+                s += r + e > j ? dabs2(t) : 0.0;
             }
+        s = warp_sum(s);
+        x.sync();
+        if (x.lane == 0) *reinterpret_cast<double*>(pn + x.h * 16) = s;
+        x.sync();
+#pragma unroll 1
+        for (int hh = 0; hh < S; ++hh) xn2 += *reinterpret_cast<const double*>(pn + hh * 16);
+    }
+    T tau = tzero<T>(), scale = tzero<T>(), beta = alpha;
+    bool done = false;
+    if constexpr (!is_complex_v<T>) {
+        // short chain: float32 on the float-float sum alpha^2 + |x|^2, float64 where
+        // the sum is in float32's range
+        T a2;
+        bool ok;
+        if constexpr (sizeof(T) == 4) {
+            a2 = nrm.plus_square(alpha);
+            ok = !tiny;
+        } else {
+            a2 = fma(alpha, alpha, nrm.value());
+            ok = qr_in_range(nrm.value(), a2);
+        }
+        if (ok) {
+            if (sizeof(T) == 8 || nrm.value() > T(0)) {
+                T nr, quo, inv;
+                qr_scalars(a2, alpha < T(0) ? -alpha : alpha, nr, quo, inv);
+                beta = tcopysign(nr, alpha);
+                beta = -beta;
+                tau = quo;
+                scale = tcopysign(inv, alpha);
+            }
+            done = true;
         }
     }
-    __syncthreads();
-    for (int j = 0; j < pw; ++j) {
-        T* x = P + j * ldp;
-        if (tid == 0) {
-            int k = j;
-            if (piv) {
-                RT best = met[j];
-                for (int c = j + 1; c < pw; ++c)
-                    if (met[c] > best) {
-                        best = met[c];
-                        k = c;
-                    }
-                if (k != j) {
-                    const int ti = pmp[j];
-                    pmp[j] = pmp[k];
-                    pmp[k] = ti;
-                    const double tn = nb2[j];
-                    nb2[j] = nb2[k];
-                    nb2[k] = tn;
-                }
-                ksh = k;
-            }
-            T* xk = P + k * ldp;  // the column that becomes column j
-            const double xn2 = piv ? nb2[j] : red[j & 1];
-            const T alpha = xk[j];
-            T tau = tzero<T>(), scale = tzero<T>();
-            const double a2 = dabs2(alpha) + xn2;
-            // a sub-column below (1e-30)^2 (float32) is treated as zero
-            if (xn2 > 0.0 && a2 > (sizeof(RT) == 4 ? 1e-60 : 0.0)) {
-                if constexpr (is_complex_v<T>) {
-                    // beta = -sign(Re alpha) |(alpha, x)| (real), tau = (beta - alpha) / beta,
-                    // scale = 1 / (alpha - beta), evaluated in float64
-                    const double ar = alpha.x, ai = alpha.y;
-                    const double beta = -copysign(sqrt(a2), ar);
-                    tau = T{RT((beta - ar) / beta), RT(-ai / beta)};
-                    const double zr = ar - beta, zi = ai, zz = zr * zr + zi * zi;
+    if (!done) {
+        if (!tiny) xn2 = nrm.wide();
+        const double a2 = dabs2(alpha) + xn2;
+        // a sub-column below (1e-30)^2 (float32) is treated as zero
+        if (xn2 > 0.0 && a2 > (sizeof(RT) == 4 ? 1e-60 : 0.0)) {
+            if constexpr (is_complex_v<T>) {
+                // beta = -sign(Re alpha) |(alpha, x)| (real), tau = (beta - alpha) / beta,
+                // scale = 1 / (alpha - beta), evaluated in float64
+                const double ar = alpha.x, ai = alpha.y;
+                if (qr_in_range(xn2, a2)) {
+                    double r;
+                    const double nr = qr_root(a2, r), ab = fabs(ar), zr = ab + nr;
+                    const double quo = zr * r, iz = qr_recip(fma(zr, zr, ai * ai));
+                    tau = T{RT(fma(r, fma(-quo, nr, zr), quo)), RT(copysign(1.0, ar) * ai * r)};
+                    scale = T{RT(copysign(zr * iz, ar)), RT(-ai * iz)};
+                    beta = T{RT(-copysign(nr, ar)), RT(0)};
+                } else {
+                    const double bt = -copysign(sqrt(a2), ar);
+                    tau = T{RT((bt - ar) / bt), RT(-ai / bt)};
+                    const double zr = ar - bt, zi = ai, zz = zr * zr + zi * zi;
                     scale = T{RT(zr / zz), RT(-zi / zz)};
-                    xk[j] = T{RT(beta), RT(0)};
-                } else if (sizeof(T) == 4 && a2 >= 1e-36) {
-                    const T beta = -tcopysign(tsqrt(T(a2)), alpha);
-                    tau = (beta - alpha) / beta;
-                    scale = T(1) / (alpha - beta);
-                    xk[j] = beta;
-                } else {  // float64 (and float32 columns too small for float32 arithmetic)
-                    const double al = alpha;
-                    const double beta = -copysign(sqrt(a2), al);
-                    tau = T((beta - al) / beta);
-                    scale = T(1.0 / (al - beta));
-                    xk[j] = T(beta);
+                    beta = T{RT(bt), RT(0)};
                 }
-            }
-            Tm[j * nb + j] = tau;
-            psc[j] = scale;
-        }
-        __syncthreads();
-        if (piv) {
-            const int k = ksh;
-            if (k != j) {
-                T* xk = P + k * ldp;
-                for (int r = tid; r < R4; r += nt) {
-                    const T t = x[r];
-                    x[r] = xk[r];
-                    xk[r] = t;
-                }
+            } else {
+                const double al = alpha;
+                const double bt = -copysign(sqrt(a2), al);
+                tau = T((bt - al) / bt);
+                scale = T(1.0 / (al - bt));
+                beta = T(bt);
             }
         }
-        const T tau = Tm[j * nb + j], scale = psc[j];
-        if (j > 0) {
-            const T sp = psc[j - 1];
-            T* xp = P + (j - 1) * ldp;
-            for (int r = j + tid; r < R; r += nt) xp[r] *= sp;
-        }
-        if (piv) __syncthreads();
-        for (int c = j + 1 + wid; c < pw; c += nw) {
-            T* y = P + c * ldp;
-            if (tau != tzero<T>()) {
-                // x is scaled inside the dot: the product of two raw sub-columns
-                // would underflow in float32 for entries below ~1e-19.
-                // y <- H^H y = y - conj(tau) v (v^H y), v = (1, x scale)
-                T s0 = tzero<T>(), s1 = tzero<T>();
-                int r = j + 1 + lane;
-                for (; r + 32 < R; r += 64) {
-                    s0 += tconj_mul(x[r] * scale, y[r]);
-                    s1 += tconj_mul(x[r + 32] * scale, y[r + 32]);
-                }
-                if (r < R) s0 += tconj_mul(x[r] * scale, y[r]);
-                const T sdot = warp_sum(s0 + s1) + y[j];
-                const T f = tconj(tau) * sdot, fs = f * scale;
-                for (int rr = j + 1 + lane; rr < R; rr += 32) y[rr] -= fs * x[rr];
-                __syncwarp();
-                if (lane == 0) y[j] -= f;
-            }
-            if (piv) {
-                __syncwarp();
-                const double t = col_norm2(y, j + 2, R);
-                if (lane == 0) {
-                    nb2[c] = t;
-                    met[c] = RT(dabs2(y[j + 1]) + t);
-                }
-            } else if (c == j + 1) {
-                __syncwarp();
-                const double t = col_norm2(y, j + 2, R);
-                if (lane == 0) red[(j + 1) & 1] = t;
-            }
-        }
-        __syncthreads();
     }
-    {
-        const int j = pw - 1;
-        const T sp = psc[j];
-        T* xp = P + j * ldp;
-        for (int r = j + 1 + tid; r < R; r += nt) xp[r] *= sp;
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+        T v[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            v[e] = y[q][e] * scale;
+            if (q == 0) {  // rows at and above j lie in the first chunk of warp 0
+                const int r = x.row(0) + e;
+                if (r <= j) v[e] = r == j ? tone<T>() : tzero<T>();
+                y[0][e] = r > j ? v[e] : (r == j ? beta : y[0][e]);
+            } else {
+                y[q][e] = v[e];
+            }
+        }
+        qr_st(x.P + j * x.ldp + x.row(q), v);
     }
-    __syncthreads();
+    if (x.h == 0 && x.lane == 0) x.Tm[j * x.LDT + j] = tau;
 }
 
-// T of the compact WY form of the panel (explicit V in P, tau_j on Tm's
-// diagonal): G = V^H V with the tiled product, then row i of T by one lane:
-// T[i][j] = -tau_j sum_{l=i}^{j-1} T[i][l] G[l][j] for j > i (the columnwise
-// recursion of Schreiber & Van Loan, read by rows), zeros below the diagonal.
-template <class T, int NI>
-__device__ void qr_t_matrix(const T* P, int ldp, int R, int pw, T* Tm, int nb, T* G, T* Wp) {
-    for (int cb = 0; cb < pw; cb += QR_QG) {
-        auto col = [&](int c) -> const T* { return cb + c < pw ? P + (cb + c) * ldp : nullptr; };
-        qr_vty<T, NI>(P, ldp, pw, R, Wp, col, true);
-        __syncthreads();
-        const int nw = blockDim.x >> 5;
-        for (int o = threadIdx.x; o < pw * QR_QG; o += blockDim.x) {
-            const int i = o / QR_QG, c = o % QR_QG;
-            if (cb + c < pw) {
+// Order of a non-negative metric as an integer (NaN and negative values last).
+__device__ __forceinline__ int qr_metric_key(float v) { return v >= 0.f ? __float_as_int(v) : -1; }
+__device__ __forceinline__ int qr_metric_key(double v) { return v >= 0.0 ? __double2hiint(v) : -1; }
+
+// T of the compact WY form from tau on its diagonal and G = V^H V: with the
+// columns in two halves, T = [T1, -T1 G12 T2; 0, T2], so blocks of 1, 2, 4, ...
+// columns are joined pairwise by all threads (T is zero on entry but for its
+// diagonal; X = G12 T2 is kept below T's diagonal, which is cleared at the end).
+template <class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_t_matrix(const QrCtx<T, NB, S, NQ>& x, int pw) {
+    constexpr int LDT = NB + 1;
+    const int tid = (x.grp * S + x.h) * 32 + x.lane, nt = 32 * S * (NB / QR_NC);
+#pragma unroll 1
+    for (int b = 1; b < pw; b *= 2) {
+        // element o: pair o / b^2, row i and column j of its b x b off-diagonal block
+        for (int o = tid; o < NB / 2 * b; o += nt) {
+            const int pr = o / (b * b), e = o - pr * b * b, i = e / b, j = e - i * b;
+            const int r0 = 2 * b * pr, c0 = r0 + b;
+            if (c0 + j < pw) {
                 T s = tzero<T>();
-                for (int w = 0; w < nw; ++w) s += Wp[w * 8 * NI * QR_QG + o];
-                G[i * pw + cb + c] = s;
+                for (int l = 0; l <= j; ++l) s += x.G[(r0 + i) * LDT + c0 + l] * x.Tm[(c0 + l) * LDT + c0 + j];
+                x.Tm[(c0 + j) * LDT + r0 + i] = s;  // X, transposed into the lower block
+            }
+        }
+        __syncthreads();
+        for (int o = tid; o < NB / 2 * b; o += nt) {
+            const int pr = o / (b * b), e = o - pr * b * b, i = e / b, j = e - i * b;
+            const int r0 = 2 * b * pr, c0 = r0 + b;
+            if (c0 + j < pw) {
+                T s = tzero<T>();
+                for (int l = i; l < b; ++l) s += x.Tm[(r0 + i) * LDT + r0 + l] * x.Tm[(c0 + j) * LDT + r0 + l];
+                x.Tm[(r0 + i) * LDT + c0 + j] = tzero<T>() - s;
             }
         }
         __syncthreads();
     }
-    if (threadIdx.x < pw) {
-        const int i = threadIdx.x;
-        for (int j = 0; j < i; ++j) Tm[i * nb + j] = tzero<T>();
-        for (int j = i + 1; j < pw; ++j) {
-            T s = tzero<T>();
-            for (int l = i; l < j; ++l) s += Tm[i * nb + l] * G[l * pw + j];
-            Tm[i * nb + j] = tzero<T>() - Tm[j * nb + j] * s;
-        }
+    for (int o = tid; o < pw * pw; o += nt) {
+        const int i = o / pw, j = o - i * pw;
+        if (j < i) x.Tm[i * LDT + j] = tzero<T>();
     }
     __syncthreads();
 }
 
-template <class T>
-__device__ __forceinline__ void qr_block_apply_nb(T* A, int ld, int m, int p0, int pw, int c_begin, int c_end,
-                                                  const T* P, int ldp, const T* Tm, int nbT, T* Wp, T* W0, T* W1,
-                                                  bool transpose, const int* cm, bool vec) {
-    const int ni = qr_ni(nbT);
-    if (ni == 4)
-        qr_block_apply<T, 4>(A, ld, m, p0, pw, c_begin, c_end, P, ldp, Tm, nbT, Wp, W0, W1, transpose, cm, vec);
-    else if (ni == 2)
-        qr_block_apply<T, 2>(A, ld, m, p0, pw, c_begin, c_end, P, ldp, Tm, nbT, Wp, W0, W1, transpose, cm, vec);
-    else
-        qr_block_apply<T, 1>(A, ld, m, p0, pw, c_begin, c_end, P, ldp, Tm, nbT, Wp, W0, W1, transpose, cm, vec);
+// Householder factorisation of the panel: group g holds columns 4 g .. 4 g + 3
+// of the pw panel columns in y (R rows).  Per step: the owner forms the
+// reflector (qr_reflect), one CTA barrier, then every group takes the dots of
+// v with its four columns and updates those not yet done; the dots with
+// finished columns are the entries of G = V^H V, which give T at the end.  Pivoting (met != null): step j
+// takes the remaining column with the largest metric (its squared norm at the
+// start of the panel, reduced by the squares of the R entries found since);
+// stp[c] is the step at which this group's column c was taken.
+template <int NA, bool PIV, class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_panel(const QrCtx<T, NB, S, NQ>& x, QrQuad<T, NQ>& y, int pw, bool want_t,
+                                         real_t<T>* met, int (&stp)[QR_NC]) {
+    constexpr int V = QrVec<T>::V;
+#pragma unroll
+    for (int c = 0; c < QR_NC; ++c) stp[c] = NB;
+#pragma unroll 1
+    for (int j = 0; j < pw; ++j) {
+        int k = j;
+        if (PIV) {
+            const int key = x.lane < pw ? (met[x.lane] == real_t<T>(-2) ? -2 : qr_metric_key(met[x.lane])) : -2;
+            const int best = __reduce_max_sync(0xffffffffu, key);
+            k = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+        }
+        const int kc = x.grp == (k >> 2) ? (k & 3) : -1;  // the column of this quad that is taken
+        if (kc >= 0) {
+            // one copy of the code for the four columns: the step has to stay within
+            // the instruction cache
+            T z[NQ][V];
+            auto take = [&](auto cc) {  // compile-time column: y stays in registers
+                constexpr int c = decltype(cc)::value;
+#pragma unroll
+                for (int q = 0; q < NA; ++q)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) z[q][e] = y[c][q][e];
+            };
+            auto give = [&](auto cc) {
+                constexpr int c = decltype(cc)::value;
+                stp[c] = j;
+#pragma unroll
+                for (int q = 0; q < NA; ++q)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) y[c][q][e] = z[q][e];
+            };
+            switch (kc) {
+                case 0: take(std::integral_constant<int, 0>{}); break;
+                case 1: take(std::integral_constant<int, 1>{}); break;
+                case 2: take(std::integral_constant<int, 2>{}); break;
+                default: take(std::integral_constant<int, 3>{}); break;
+            }
+            qr_reflect<NA>(x, z, j);
+            switch (kc) {
+                case 0: give(std::integral_constant<int, 0>{}); break;
+                case 1: give(std::integral_constant<int, 1>{}); break;
+                case 2: give(std::integral_constant<int, 2>{}); break;
+                default: give(std::integral_constant<int, 3>{}); break;
+            }
+        }
+        __syncthreads();
+        if (PIV && kc >= 0 && x.h == 0 && x.lane == 0) met[k] = real_t<T>(-2);
+        // a group whose columns are all done has only its entries of G left to give
+        const bool live = max(max(stp[0], stp[1]), max(stp[2], stp[3])) == NB || want_t;
+        if (x.grp * QR_NC < pw && live) {
+            const T tau = x.Tm[j * x.LDT + j];
+            T v[NA][V];
+            QrAcc<T> acc[QR_NC];
+#pragma unroll
+            for (int q = 0; q < NA; ++q) qr_ld(v[q], x.P + j * x.ldp + x.row(q));
+#pragma unroll
+            for (int q = 0; q < NA; ++q)
+#pragma unroll
+                for (int c = 0; c < QR_NC; ++c) acc[c].add(v[q], y[c][q]);
+            T w[QR_NC];
+#pragma unroll
+            for (int c = 0; c < QR_NC; ++c) w[c] = acc[c].total();
+            const T t = qr_reduce_scatter<QR_NC>(w);
+            if constexpr (S == 1) {
+#pragma unroll
+                for (int c = 0; c < QR_NC; ++c) w[c] = shfl(t, 8 * c);
+            } else {
+                T* pd = x.pd + ((j & 1) * x.WARPS + x.grp * S) * QR_NC;
+                if ((x.lane & 7) == 0) pd[x.h * QR_NC + (x.lane >> 3)] = t;
+                x.sync();
+#pragma unroll
+                for (int c = 0; c < QR_NC; ++c) w[c] = pd[c];
+#pragma unroll
+                for (int hh = 1; hh < S; ++hh)
+#pragma unroll
+                    for (int c = 0; c < QR_NC; ++c) w[c] += pd[hh * QR_NC + c];
+            }
+            // y -= conj(tau) (v^H y) v on the columns not yet taken (factor 0 on the others)
+            const T ntau = tzero<T>() - tconj(tau);
+#pragma unroll
+            for (int c = 0; c < QR_NC; ++c) {
+                const T f = stp[c] == NB ? ntau * w[c] : tzero<T>();
+                if (sizeof(real_t<T>) == 8 && stp[c] != NB) continue;  // float64 work is scarce
+#pragma unroll
+                for (int q = 0; q < NA; ++q) qr_axpy(y[c][q], v[q], f);
+            }
+            if (x.h == 0) {
+                if (want_t) {  // dots with the finished columns: row stp[c] of G
+                    T g = w[0];
+                    int row = stp[0];
+#pragma unroll
+                    for (int c = 1; c < QR_NC; ++c) {
+                        g = x.lane == c ? w[c] : g;
+                        row = x.lane == c ? stp[c] : row;
+                    }
+                    if (x.lane < QR_NC && row < j) x.G[row * x.LDT + j] = tconj(g);
+                }
+                if (PIV) {
+#pragma unroll
+                    for (int e = 0; e < V; ++e)
+                        if (x.row(0) + e == j) {
+#pragma unroll
+                            for (int c = 0; c < QR_NC; ++c) {
+                                const int lc = x.grp * QR_NC + c;
+                                const real_t<T> d = met[lc] - tabs2(y[c][0][e]);
+                                if (stp[c] == NB) met[lc] = d > real_t<T>(0) || d != d ? d : real_t<T>(0);
+                            }
+                        }
+                }
+            }
+        }
+        if (PIV) __syncthreads();
+    }
+    __syncthreads();
+    if (want_t) qr_t_matrix(x, pw);
 }
 
-template <class T>
-__global__ void __launch_bounds__(QR_THREADS) k_qr(QRJob<T> job) {
+template <class T, int NB, int S, int NQ, bool PIV>
+__global__ void __launch_bounds__(32 * S * NB / QR_NC, S == 1 ? 2 : 1) k_qr(QRJob<T> job) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int V = QrVec<T>::V;
+    using RT = real_t<T>;
     const int b = blockIdx.x;
-    const int m = job.m, n = job.n, ld = job.ld, nb = job.nb;
+    const int m = job.m, n = job.n, ld = job.ld;
+    constexpr int nb = NB, nt = 32 * S * NB / QR_NC;
     const int kk = min(m, n);
-    const int ldp = qr_ldp<T>(m);
     T* A = job.A + (long)b * job.strideA;
     T* Tw = job.Tw + (long)b * job.strideT;
-    const bool piv = job.pivot && job.mode == QR_R_ROWS;
-    const int tid = threadIdx.x, nt = blockDim.x, nw = nt >> 5;
+    const int tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
-    const int ni = qr_ni(nb);
-    const int cap = 8 * ni;
-    double* red = reinterpret_cast<double*>(smem_raw);
-    T* P = reinterpret_cast<T*>(smem_raw + 64 * sizeof(double));
-    T* Tm = P + (size_t)nb * ldp;
-    T* G = Tm + nb * nb;
-    T* Wp = G + nb * nb;
-    T* W0 = Wp + (size_t)nw * cap * QR_QG;
-    T* W1 = W0 + (size_t)cap * QR_QG;
-    using RT = real_t<T>;
-    double* nb2 = reinterpret_cast<double*>(W1 + (size_t)cap * QR_QG);
-    RT* met = reinterpret_cast<RT*>(nb2 + nb);
+    QrCtx<T, NB, S, NQ> x;
+    x.ldp = qr_ldp<T>(m, S, NQ);
+    x.grp = wid / S;
+    x.h = wid % S;
+    x.lane = lane;
+    x.pn = smem_raw;
+    x.pa = smem_raw + 2 * x.WARPS * 16;
+    x.P = reinterpret_cast<T*>(x.pa + x.WARPS * 16);
+    x.pd = x.P + (size_t)nb * x.ldp;
+    T* grp0 = x.pd + 2 * x.WARPS * QR_NC;
+    x.W1 = grp0 + x.grp * x.GSZ;
+    x.Wp = x.W1 + QR_NC * nb;
+    x.Tm = grp0 + x.NG * x.GSZ;
+    x.G = x.Tm + nb * (nb + 4);
+    RT* met = reinterpret_cast<RT*>(x.G + nb * (nb + 4));
     RT* cnrm = met + nb;
     int* pm = reinterpret_cast<int*>(cnrm + n);
     int* pm2 = pm + n;
-    // the column map in shared memory: the given one, or the order pivoting chooses
-    {
-        const int* cin = job.colmap ? job.colmap + (long)b * n : nullptr;
-        for (int c = tid; c < n; c += nt) pm[c] = (cin && !piv) ? cin[c] : c;
-    }
-    __syncthreads();
-    const int* cm = pm;
-    // 16-byte accesses to columns of A (rows p0 + r, r a multiple of 4)
-    const bool vec = ((reinterpret_cast<uintptr_t>(A) & 15) == 0) && (ld % 4 == 0);
+    auto phys = [&](int c) { return PIV ? pm[c] : c; };
 
+    if (PIV) {  // identity order and the columns' squared norms
+        for (int c = tid; c < n; c += nt) pm[c] = c;
+        for (int c = wid; c < n; c += x.WARPS) {
+            const T* col = A + (long)c * ld;
+            RT s2 = RT(0);
+            for (int r = lane; r < m; r += 32) s2 += tabs2(col[r]);
+            s2 = warp_sum(s2);
+            if (lane == 0) cnrm[c] = s2;
+        }
+        __syncthreads();
+    }
+
+    QrQuad<T, NQ> y;
+    T* col[QR_NC];
+#pragma unroll 1
     for (int p0 = 0; p0 < kk; p0 += nb) {
         const int pw = min(nb, kk - p0);
         const int R = m - p0;
-        const int R4 = 4 * ceil_div(R, 4);
-        if (piv) {
+        if (PIV) {
             // block pivoting: order the remaining columns by their norm below row
             // p0 (ties by position; non-finite norms last), so the panel takes the
             // largest ones
-            for (int c = p0 + wid; c < n; c += nw) {
-                const T* col = A + (long)pm[c] * ld + p0;
-                RT s2 = RT(0);
-                for (int r = lane; r < R; r += 32) s2 += tabs2(col[r]);
-                s2 = warp_sum(s2);
-                if (lane == 0) cnrm[c] = (s2 == s2) ? s2 : RT(-1);
-            }
-            __syncthreads();
             for (int c = p0 + tid; c < n; c += nt) {
-                const RT v = cnrm[c];
+                RT v = cnrm[c];
+                if (!(v == v)) v = RT(-1);
                 int rank = 0;
                 for (int q = p0; q < n; ++q) {
-                    const RT w = cnrm[q];
+                    RT w = cnrm[q];
+                    if (!(w == w)) w = RT(-1);
                     rank += (w > v) || (w == v && q < c);
                 }
                 pm2[p0 + rank] = pm[c];
+                if (rank < pw) met[rank] = v;
             }
             __syncthreads();
             for (int c = p0 + tid; c < n; c += nt) pm[c] = pm2[c];
             __syncthreads();
         }
-        for (int i = tid; i < pw * R4; i += nt) {
-            const int c = i / R4, r = i % R4;
-            P[c * ldp + r] = r < R ? A[(long)QCOL(p0 + c) * ld + p0 + r] : tzero<T>();
+        int lc[QR_NC], stp[QR_NC];
+#pragma unroll
+        for (int c = 0; c < QR_NC; ++c) {
+            const int l = x.grp * QR_NC + c;
+            lc[c] = l < pw ? phys(p0 + l) : -1;
+            col[c] = l < pw ? A + (long)lc[c] * ld + p0 : nullptr;
         }
+        qr_load<T, NB, S, NQ>(x, y, col, R);
+        for (int o = tid; o < nb * x.LDT; o += nt) x.Tm[o] = tzero<T>();
         __syncthreads();
-        qr_panel(P, ldp, R, pw, Tm, nb, W0, red, piv ? pm + p0 : nullptr, nb2, met);
-        // write the factored panel (R above, reflectors below the diagonal) back
-        for (int i = tid; i < pw * R; i += nt) {
-            const int c = i / R, r = i % R;
-            A[(long)QCOL(p0 + c) * ld + p0 + r] = P[c * ldp + r];
+        const bool want_t = !PIV || p0 + pw < n;
+        const bool full = qr_active(R, V, S, NQ) == NQ;
+        if (full) qr_panel<NQ, PIV>(x, y, pw, want_t, met, stp);
+        else qr_panel<NQ / 2, PIV>(x, y, pw, want_t, met, stp);
+        // the factored panel (R above, reflectors below the diagonal) back to A
+        qr_store<T, NB, S, NQ>(x, y, col, R);
+        if (PIV && x.h == 0 && lane == 0) {
+#pragma unroll
+            for (int c = 0; c < QR_NC; ++c)
+                if (lc[c] >= 0) pm[p0 + stp[c]] = lc[c];
         }
-        __syncthreads();
-        qr_explicit_v(P, ldp, pw);
-        __syncthreads();
-        if (ni == 4) qr_t_matrix<T, 4>(P, ldp, R, pw, Tm, nb, G, Wp);
-        else if (ni == 2) qr_t_matrix<T, 2>(P, ldp, R, pw, Tm, nb, G, Wp);
-        else qr_t_matrix<T, 1>(P, ldp, R, pw, Tm, nb, G, Wp);
-        // keep T for forming Q
-        for (int i = tid; i < nb * nb; i += nt) Tw[(p0 / nb) * nb * nb + i] = Tm[i];
-        // --- trailing update of columns p0+pw .. n-1
-        if (p0 + pw < n)
-            qr_block_apply_nb<T>(A, ld, m, p0, pw, p0 + pw, n, P, ldp, Tm, nb, Wp, W0, W1, true, cm, vec);
+        // T for forming or applying Q
+        if (!PIV)
+            for (int o = tid; o < nb * nb; o += nt) Tw[(long)(p0 / nb) * nb * nb + o] = x.Tm[(o / nb) * x.LDT + o % nb];
+        // --- trailing update of columns p0+pw .. n-1, a quad per group
+#pragma unroll 1
+        for (int c0 = p0 + pw + QR_NC * x.grp; c0 < n; c0 += QR_NC * x.NG) {
+#pragma unroll
+            for (int c = 0; c < QR_NC; ++c) col[c] = c0 + c < n ? A + (long)phys(c0 + c) * ld + p0 : nullptr;
+            qr_load<T, NB, S, NQ>(x, y, col, R);
+            if (full) qr_apply_quad<NQ>(x, y, pw, true);
+            else qr_apply_quad<NQ / 2>(x, y, pw, true);
+            qr_store<T, NB, S, NQ>(x, y, col, R);
+            if (PIV) {  // their norms below row p0 + pw, for the next panel
+                RT s2[QR_NC];
+#pragma unroll
+                for (int c = 0; c < QR_NC; ++c) {
+                    s2[c] = RT(0);
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                        for (int e = 0; e < V; ++e)
+                            if (x.row(q) + e >= pw) s2[c] += tabs2(y[c][q][e]);
+                }
+                const RT t = qr_reduce_scatter<QR_NC>(s2);
+                RT* pd = reinterpret_cast<RT*>(x.pd + x.grp * S * QR_NC);
+                if ((lane & 7) == 0) pd[x.h * QR_NC + (lane >> 3)] = t;
+                x.sync();
+                if (x.h == 0 && lane < QR_NC && c0 + lane < n) {
+                    RT s = RT(0);
+#pragma unroll 1
+                    for (int hh = 0; hh < S; ++hh) s += pd[hh * QR_NC + lane];
+                    cnrm[c0 + lane] = s;
+                }
+            }
+        }
         __syncthreads();
     }
 
     // --- outputs
     T* out = job.out + (long)b * job.strideOut;
-    if (job.mode == QR_R_ROWS) {
+    if constexpr (PIV) {
         for (int i = tid; i < n * n; i += nt) {
             const int r = i / n, c = i % n;
-            out[i] = (r <= c && r < kk) ? A[(long)QCOL(c) * ld + r] : tzero<T>();
+            out[i] = (r <= c && r < kk) ? A[(long)phys(c) * ld + r] : tzero<T>();
         }
-        if (piv)
-            for (int c = tid; c < n; c += nt) job.colmap[(long)b * n + c] = pm[c];
-        return;
-    }
-    // QR_L_AND_Q / QR_L_ONLY: L = R^T (n x kk)
-    for (int i = tid; i < n * kk; i += nt) {
-        const int r = i / kk, c = i % kk;
-        out[i] = (c <= r) ? A[(long)QCOL(r) * ld + c] : tzero<T>();
-    }
-    if (job.mode == QR_L_ONLY) return;
-    __syncthreads();
-    // form Q in place, panels in reverse order
-    const int npan = ceil_div(kk, nb);
-    for (int pi = npan - 1; pi >= 0; --pi) {
-        const int p0 = pi * nb;
-        const int pw = min(nb, kk - p0);
-        const int R = m - p0;
-        const int R4 = 4 * ceil_div(R, 4);
-        for (int i = tid; i < pw * R4; i += nt) {
-            const int c = i / R4, r = i % R4;
-            P[c * ldp + r] = r < R ? A[(long)QCOL(p0 + c) * ld + p0 + r] : tzero<T>();
+        for (int c = tid; c < n; c += nt) job.colmap[(long)b * n + c] = pm[c];
+    } else {
+        // QR_L_AND_Q / QR_L_ONLY: L = R^T (n x kk)
+#pragma unroll 4
+        for (int i = tid; i < n * kk; i += nt) {
+            const int r = i / kk, c = i % kk;
+            out[i] = (c <= r) ? A[(long)r * ld + c] : tzero<T>();
         }
-        for (int i = tid; i < nb * nb; i += nt) Tm[i] = Tw[pi * nb * nb + i];
+        if (job.mode == QR_L_ONLY) return;
         __syncthreads();
-        qr_explicit_v(P, ldp, pw);
-        __syncthreads();
-        if (p0 + pw < kk)
-            qr_block_apply_nb<T>(A, ld, m, p0, pw, p0 + pw, kk, P, ldp, Tm, nb, Wp, W0, W1, false, cm, vec);
-        qr_form_panel<T>(A, ld, m, p0, pw, P, ldp, Tm, nb, W0, W1, cm, vec);
+        // form Q in place, panels in reverse order: the panel's block reflector on the
+        // later columns of Q and on the identity columns of its own
+#pragma unroll 1
+        for (int pi = (kk - 1) / nb; pi >= 0; --pi) {
+            const int p0 = pi * nb;
+            const int pw = min(nb, kk - p0);
+            const int R = m - p0;
+            const bool full = qr_active(R, V, S, NQ) == NQ;
+            for (int o = tid; o < pw * x.ldp; o += nt) {
+                const int i = o / x.ldp, r = o % x.ldp;
+                x.P[o] = r < i || r >= R ? tzero<T>() : (r == i ? tone<T>() : A[(long)(p0 + i) * ld + p0 + r]);
+            }
+            for (int o = tid; o < nb * nb; o += nt) x.Tm[(o / nb) * x.LDT + o % nb] = Tw[(long)pi * nb * nb + o];
+            __syncthreads();
+#pragma unroll 1
+            for (int c0 = p0 + QR_NC * x.grp; c0 < kk; c0 += QR_NC * x.NG) {
+                const bool own = c0 < p0 + pw;
+#pragma unroll
+                for (int c = 0; c < QR_NC; ++c) col[c] = c0 + c < kk ? A + (long)(c0 + c) * ld + p0 : nullptr;
+                if (own) {
+#pragma unroll
+                    for (int c = 0; c < QR_NC; ++c)
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                            for (int e = 0; e < V; ++e)
+                                y[c][q][e] = x.row(q) + e == c0 + c - p0 ? tone<T>() : tzero<T>();
+                } else {
+                    qr_load<T, NB, S, NQ>(x, y, col, R);
+                }
+                if (full) qr_apply_quad<NQ>(x, y, pw, false);
+                else qr_apply_quad<NQ / 2>(x, y, pw, false);
+                qr_store<T, NB, S, NQ>(x, y, col, R);
+            }
+            for (int i = tid; i < pw * p0; i += nt) A[(long)(p0 + i / p0) * ld + i % p0] = tzero<T>();
+            __syncthreads();
+        }
+    }
+}
+
+// f(kernel) for shape i of QR_SHAPES
+template <class T, bool PIV, class F>
+inline void qr_dispatch(int shape, F&& f) {
+    switch (shape) {
+        case 0: return f(k_qr<T, 32, 1, 2, PIV>);
+        case 1: return f(k_qr<T, 32, 1, 4, PIV>);
+        case 2: return f(k_qr<T, 32, 2, 4, PIV>);
+        case 3: return f(k_qr<T, 16, 4, 4, PIV>);
+        case 4: return f(k_qr<T, 8, 8, 4, PIV>);
+        default: return f(k_qr<T, 4, 16, 4, PIV>);
     }
 }
 
