@@ -353,8 +353,8 @@ struct Engine {
             // normalise U's columns, then M = diag(nu) (I - F') V with F = V V^T
             {
                 THC_LAUNCH("svd_finalize", st);
-                dim3 g(ceil_div(kout, 128), B);
-                k_unit_columns<T><<<g, 128, 0, st>>>(out + pO.off[s], out_stride, m, kout, w.nu, w.sSv);
+                dim3 g(ceil_div(kout, UC_COLS), B);
+                k_unit_columns<T><<<g, UC_COLS * UC_ROWS, 0, st>>>(out + pO.off[s], out_stride, m, kout, w.nu, w.sSv);
             }
             check();
             {

@@ -594,22 +594,38 @@ __global__ void __launch_bounds__(JacobiCfg<T, NPL>::threads) k_jacobi_select(Ja
 }
 
 // Finalisation per term, step 1: normalise the columns of U (mU x kout,
-// row-major, in place) and keep their norms nu (coalesced: thread j walks
-// column j).  Steps 2 and 3 are batched GEMMs on the engine side:
-// F = V V^T, then M = diag(nu) (I - F') V with F' = F - I on the kept rows.
+// row-major, in place) and keep their norms nu.  A CTA takes 8 columns, 32
+// threads down the rows of each (a warp reads 4 rows x 8 columns), so that a
+// column is a chain of mU / 32 steps and one matrix gives kout / 8 CTAs; bound by
+// the latency of that chain for one matrix (one thread per column took 45 us a
+// launch at 512 x 128 float32), by L2 for many.  Steps 2 and 3 are batched GEMMs
+// on the engine side: F = V V^T, then M = diag(nu) (I - F') V with F' = F - I on
+// the kept rows.
+constexpr int UC_COLS = 8, UC_ROWS = 32;
 template <class T>
-__global__ void __launch_bounds__(256) k_unit_columns(T* U, long strideU, int mU, int kout, T* nu,
-                                                      long strideNu) {
-    const int b = blockIdx.y;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= kout) return;
+__global__ void __launch_bounds__(UC_COLS* UC_ROWS) k_unit_columns(T* U, long strideU, int mU, int kout, T* nu,
+                                                                    long strideNu) {
+    __shared__ double part[UC_ROWS][UC_COLS];
+    const int b = blockIdx.y, c = threadIdx.x % UC_COLS, rl = threadIdx.x / UC_COLS;
+    const int j = blockIdx.x * UC_COLS + c;
     U += (long)b * strideU;
     double acc = 0.0;
-    for (int r = 0; r < mU; ++r) acc += (double)tabs2(U[(long)r * kout + j]);
-    const double nrm = sqrt(acc);
+    if (j < kout)
+#pragma unroll 4
+        for (int r = rl; r < mU; r += UC_ROWS) acc += (double)tabs2(U[(long)r * kout + j]);
+    part[rl][c] = acc;
+    __syncthreads();
+#pragma unroll
+    for (int o = UC_ROWS / 2; o >= 1; o >>= 1) {
+        if (rl < o) part[rl][c] += part[rl + o][c];
+        __syncthreads();
+    }
+    if (j >= kout) return;
+    const double nrm = sqrt(part[0][c]);
     const real_t<T> inv = nrm > 0.0 ? real_t<T>(1.0 / nrm) : real_t<T>(0);
-    for (int r = 0; r < mU; ++r) U[(long)r * kout + j] = tscale(U[(long)r * kout + j], inv);
-    nu[(long)b * strideNu + j] = nrm > 0.0 ? treal<T>(real_t<T>(nrm)) : tzero<T>();
+#pragma unroll 4
+    for (int r = rl; r < mU; r += UC_ROWS) U[(long)r * kout + j] = tscale(U[(long)r * kout + j], inv);
+    if (rl == 0) nu[(long)b * strideNu + j] = nrm > 0.0 ? treal<T>(real_t<T>(nrm)) : tzero<T>();
 }
 
 // A-operand of M = diag(nu) (I - F') V: element (i, l) = nu_i (delta_il - F'_il),
