@@ -70,6 +70,7 @@ static __global__ void k_set_int(int* p, int v) { *p = v; }
 
 template <class T>
 struct AdjTransA {  // A(m, k) = base_b[k*ld + m] (transposed access, real)
+    static constexpr bool walk_m = true;
     const T* base;
     long stride;
     int ld;
