@@ -16,12 +16,18 @@
 //   * Z = X V_p: warp w takes a contiguous range of quads of the K = m - p0
 //     rows of V_p; lane (rq, cq) accumulates the 8 x 4 tile rows rq + 4 i,
 //     columns 4 cq.. with 16-byte loads of X (shared) and of V's columns
-//     (global; the zero/one substitution of V's triangle only on the panel's
-//     first 32 rows); the 16 warp partials are summed in shared memory;
-//   * Z <- Z T_p^T (T upper triangular);
+//     (global, the next quad's in flight during this one's products; the
+//     zero/one substitution of V's triangle only on the panel's first 32 rows);
+//     the 16 warp partials are summed in shared memory;
+//   * Z <- Z T_p^T (T upper triangular, held at a pitch of 33: a warp reads one
+//     entry of every row of T at a time);
 //   * X[:, p0:] -= Z V_p^T: two adjacent columns of X per thread, V's rows
 //     k, k+1 read with one 8-byte load per panel column, coalesced across the
-//     warp.
+//     warp; multiply-adds on the packed pair.  With fewer than 512 (256) columns
+//     left, two (four) groups of threads share the rows.
+// Bound by the FMA pipe in the two products.  Measured, all launches of 608 terms
+// at L = 16, D = 128: 133 -> 121 ms (a pitch of 32 for T was a 16-way bank conflict;
+// no load ahead; W written a column apart; idle threads below 1024 columns).
 // Real float32 only, panels of 32 columns, m <= 1024 (the LQ-sweep shapes of
 // the float paths up to D_max = 256); other shapes form Q in the QR kernel.
 #pragma once
@@ -33,6 +39,7 @@ namespace thc {
 constexpr int QT_THREADS = 512;
 constexpr int QT_RB = 32;  // rows of X per CTA
 constexpr int QT_NB = 32;  // panel width
+constexpr int QT_LDT = QT_NB + 1;  // pitch of T in shared memory
 
 template <class T>
 struct QtJob {
@@ -57,7 +64,7 @@ __host__ __device__ inline int qt_ldx(int m) { return m + 4; }
 
 __host__ inline size_t qt_smem_bytes(int m) {
     return sizeof(float) * ((size_t)QT_RB * qt_ldx(m) + (size_t)(QT_THREADS / 32) * QT_RB * QT_NB +
-                            2 * QT_RB * QT_NB + QT_NB * QT_NB);
+                            2 * QT_RB * QT_NB + QT_NB * QT_LDT);
 }
 
 // V_p's element (row k of A, panel column j): zero above the diagonal, one on it
@@ -75,7 +82,7 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
     float* Zp = X + (size_t)QT_RB * ldx;                          // 16 warps x (QT_RB x QT_NB)
     float* Z = Zp + (size_t)(QT_THREADS / 32) * QT_RB * QT_NB;    // QT_RB x QT_NB
     float* Z2 = Z + QT_RB * QT_NB;                                // Z T^T
-    float* Tm = Z2 + QT_RB * QT_NB;                               // QT_NB x QT_NB
+    float* Tm = Z2 + QT_RB * QT_NB;                               // QT_NB x QT_LDT
     const float* M = job.M + (long)b * job.strideM;
     const float* A = job.A + (long)b * job.strideA;
     const float* Tw = job.Tw + (long)b * job.strideT;
@@ -90,7 +97,8 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
     const int np = ceil_div(kk, QT_NB);
     for (int p = np - 1; p >= 0; --p) {
         const int p0 = p * QT_NB, pw = min(QT_NB, kk - p0);
-        for (int i = tid; i < QT_NB * QT_NB; i += QT_THREADS) Tm[i] = Tw[(long)p * QT_NB * QT_NB + i];
+        for (int i = tid; i < QT_NB * QT_NB; i += QT_THREADS) 
+            Tm[i / QT_NB * QT_LDT + i % QT_NB] = Tw[(long)p * QT_NB * QT_NB + i];
         __syncthreads();
         // ---- Z = X[:, p0:m] V_p, K split over the warps in quads of rows
         {
@@ -102,15 +110,23 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
             for (int i = 0; i < 8; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+            float4 nv[4];
+            auto fetch = [&](int q) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int col = 4 * cq + j;
+                    nv[j] = col < pw && q < q1
+                                ? *reinterpret_cast<const float4*>(A + (long)(p0 + col) * job.ld + p0 + 4 * q)
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            };
+            fetch(q0);
             for (int q = q0; q < q1; ++q) {
                 const int k = p0 + 4 * q;
                 float4 v[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int col = 4 * cq + j;
-                    v[j] = col < pw ? *reinterpret_cast<const float4*>(A + (long)(p0 + col) * job.ld + k)
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                for (int j = 0; j < 4; ++j) v[j] = nv[j];
+                fetch(q + 1);
                 if (k < p0 + QT_NB) {  // the panel's triangle: zeros above the diagonal, ones on it
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -135,9 +151,8 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    Zp[(size_t)wid * QT_RB * QT_NB + (rq + 4 * i) * QT_NB + 4 * cq + j] = acc[i][j];
+                *reinterpret_cast<float4*>(Zp + (size_t)wid * QT_RB * QT_NB + (rq + 4 * i) * QT_NB + 4 * cq) =
+                    make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
         }
         __syncthreads();
         for (int o = tid; o < QT_RB * QT_NB; o += QT_THREADS) {
@@ -151,13 +166,15 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
             const int r = o / QT_NB, j = o - r * QT_NB;
             float s = 0.f;
             if (j < pw)
-                for (int i = j; i < pw; ++i) s += Z[r * QT_NB + i] * Tm[j * QT_NB + i];
+                for (int i = j; i < pw; ++i) s += Z[r * QT_NB + i] * Tm[j * QT_LDT + i];
             Z2[o] = s;
         }
         __syncthreads();
         // ---- X[:, p0:m] -= Z2 V_p^T, two adjacent columns per thread (p0 and m
         // are even): V's rows k, k+1 come with one 8-byte load per panel column
-        for (int k = p0 + 2 * tid; k < m; k += 2 * QT_THREADS) {
+        const int split = m - p0 > QT_THREADS ? 1 : m - p0 > QT_THREADS / 2 ? 2 : 4;  // groups sharing the rows
+        const int per = QT_THREADS / split, rg = tid / per;
+        for (int k = p0 + 2 * (tid - rg * per); k < m; k += 2 * per) {
             float2 v[QT_NB];
 #pragma unroll
             for (int j = 0; j < QT_NB; ++j)
@@ -171,25 +188,21 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
                 }
             }
 #pragma unroll 2
-            for (int r = 0; r < QT_RB; ++r) {
+            for (int r = rg * (QT_RB / split); r < (rg + 1) * (QT_RB / split); ++r) {
                 const float4* zr = reinterpret_cast<const float4*>(Z2 + r * QT_NB);
-                float s0 = 0.f, s1 = 0.f;
+                float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int j4 = 0; j4 < QT_NB / 4; ++j4) {
                     const float4 z = zr[j4];
-                    s0 = fmaf(z.x, v[4 * j4].x, s0);
-                    s1 = fmaf(z.x, v[4 * j4].y, s1);
-                    s0 = fmaf(z.y, v[4 * j4 + 1].x, s0);
-                    s1 = fmaf(z.y, v[4 * j4 + 1].y, s1);
-                    s0 = fmaf(z.z, v[4 * j4 + 2].x, s0);
-                    s1 = fmaf(z.z, v[4 * j4 + 2].y, s1);
-                    s0 = fmaf(z.w, v[4 * j4 + 3].x, s0);
-                    s1 = fmaf(z.w, v[4 * j4 + 3].y, s1);
+                    sum = __ffma2_rn(make_float2(z.x, z.x), v[4 * j4], sum);
+                    sum = __ffma2_rn(make_float2(z.y, z.y), v[4 * j4 + 1], sum);
+                    sum = __ffma2_rn(make_float2(z.z, z.z), v[4 * j4 + 2], sum);
+                    sum = __ffma2_rn(make_float2(z.w, z.w), v[4 * j4 + 3], sum);
                 }
                 float2* xr = reinterpret_cast<float2*>(X + (size_t)r * ldx + k);
                 float2 x = *xr;
-                x.x -= s0;
-                x.y -= s1;
+                x.x -= sum.x;
+                x.y -= sum.y;
                 *xr = x;
             }
         }
@@ -203,10 +216,12 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
         // W viewed as (4 out) x nW column-major; m = 4 nW
         float* W = job.W + (long)b * job.strideW;
         const int mW = 4 * job.out;
-        for (int r = 0; r < rows; ++r)
-            for (int qb = 0; qb < 4; ++qb)
-                for (int j = tid; j < job.nW; j += QT_THREADS)
-                    W[(long)j * mW + (r0 + r) * 4 + qb] = X[(size_t)r * ldx + qb * job.nW + j];
+        // (r, qb) fastest: a column of W gets 4 rows contiguous floats
+        for (int i = tid; i < QT_RB * 4 * job.nW; i += QT_THREADS) {
+            const int rb = i % (QT_RB * 4), j = i / (QT_RB * 4);
+            if (rb < 4 * rows)
+                W[(long)j * mW + r0 * 4 + rb] = X[(size_t)(rb >> 2) * ldx + (rb & 3) * job.nW + j];
+        }
     }
 }
 
