@@ -140,7 +140,7 @@ def svd_flops(m, n):
 UNIT_OF = {"qr_lq_sweep": "qr", "qr_svd_precond": "svd", "jacobi_svd": "svd", "gemm_expand_absorb": "gemm",
            "gemm_center": "gemm", "qt_apply": "gemm", "gemm_u": "gemm", "svd_finalize": "gemm"}
 KERNELS_OF = {"qr": "k_qr (LQ sweep launches)", "svd": "k_qr (pivoted R-only launches) + k_jacobi_select",
-              "gemm": "k_gemm128 / k_gemm / k_gemm_tc / k_apply_qt"}
+              "gemm": "k_gemm_tile / k_gemm_small / k_gemm_tc / k_apply_qt"}
 
 
 def flop_models(w, D, n_applied=None):

@@ -25,7 +25,8 @@
 //     k, k+1 read with one 8-byte load per panel column, coalesced across the
 //     warp; multiply-adds on the packed pair.  With fewer than 512 (256) columns
 //     left, two (four) groups of threads share the rows.
-// Bound by the FMA pipe in the two products.  Measured, all launches of 608 terms
+// Bound by load latency and issue (one CTA of 16 warps per SM; about six times the
+// FMA time of its products).  Measured, all launches of 608 terms
 // at L = 16, D = 128: 133 -> 121 ms (a pitch of 32 for T was a 16-way bank conflict;
 // no load ahead; W written a column apart; idle threads below 1024 columns).
 // Real float32 only, panels of 32 columns, m <= 1024 (the LQ-sweep shapes of
