@@ -16,7 +16,8 @@
 //   * Z = X V_p: warp w takes a contiguous range of quads of the K = m - p0
 //     rows of V_p; lane (rq, cq) accumulates the 8 x 4 tile rows rq + 4 i,
 //     columns 4 cq.. with 16-byte loads of X (shared) and of V's columns
-//     (global, the next quad's in flight during this one's products; the
+//     (global, loaded 8 quads ahead, a warp
+//     at a time in full lines, and staged in the space of its partial sums; the
 //     zero/one substitution of V's triangle only on the panel's first 32 rows);
 //     the 16 warp partials are summed in shared memory;
 //   * Z <- Z T_p^T (T upper triangular, held at a pitch of 33: a warp reads one
@@ -25,10 +26,12 @@
 //     k, k+1 read with one 8-byte load per panel column, coalesced across the
 //     warp; multiply-adds on the packed pair.  With fewer than 512 (256) columns
 //     left, two (four) groups of threads share the rows.
-// Bound by load latency and issue (one CTA of 16 warps per SM; about six times the
-// FMA time of its products).  Measured, all launches of 608 terms
-// at L = 16, D = 128: 133 -> 121 ms (a pitch of 32 for T was a 16-way bank conflict;
-// no load ahead; W written a column apart; idle threads below 1024 columns).
+// Bound by shared-memory reads and issue beside the FMA pipe (one CTA of 16 warps
+// per SM).  Measured: 608 x (m = 1024, kk = 256, out = 128) 4.05 -> 3.05 ms when V was
+// staged (a lane reading V's columns directly used half of each 32-byte sector);
+// all launches of 608 terms at L = 16, D = 128: 133 -> 121 ms by T's pitch (32 was a
+// 16-way bank conflict), loads ahead, W written along its columns and row groups in
+// narrow updates, -> 93 ms by the staging.
 // Real float32 only, panels of 32 columns, m <= 1024 (the LQ-sweep shapes of
 // the float paths up to D_max = 256); other shapes form Q in the QR kernel.
 #pragma once
@@ -69,7 +72,7 @@ __host__ inline size_t qt_smem_bytes(int m) {
 }
 
 // V_p's element (row k of A, panel column j): zero above the diagonal, one on it
-__device__ __forceinline__ float qt_v(const float* A, int ld, int p0, int j, int k, float loaded) {
+__device__ __forceinline__ float qt_v(int p0, int j, int k, float loaded) {
     const int kr = k - p0;
     return kr < j ? 0.f : (kr == j ? 1.f : loaded);
 }
@@ -98,7 +101,7 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
     const int np = ceil_div(kk, QT_NB);
     for (int p = np - 1; p >= 0; --p) {
         const int p0 = p * QT_NB, pw = min(QT_NB, kk - p0);
-        for (int i = tid; i < QT_NB * QT_NB; i += QT_THREADS) 
+        for (int i = tid; i < QT_NB * QT_NB; i += QT_THREADS)
             Tm[i / QT_NB * QT_LDT + i % QT_NB] = Tw[(long)p * QT_NB * QT_NB + i];
         __syncthreads();
         // ---- Z = X[:, p0:m] V_p, K split over the warps in quads of rows
@@ -111,45 +114,53 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
             for (int i = 0; i < 8; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-            float4 nv[4];
-            auto fetch = [&](int q) {
+            // V's next 8 quads of rows: a warp's load covers 32 rows of 4 columns; staged
+            // in the warp's own part of Zp with the row quad XORed by column / 4
+            float4* Vs = reinterpret_cast<float4*>(Zp + (size_t)wid * QT_RB * QT_NB);
+            const int lc = lane >> 3, lq = lane & 7;
+            float4 nv[8];
+            auto fetch = [&](int qc) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int col = 4 * cq + j;
-                    nv[j] = col < pw && q < q1
-                                ? *reinterpret_cast<const float4*>(A + (long)(p0 + col) * job.ld + p0 + 4 * q)
+                for (int i = 0; i < 8; ++i)
+                    nv[i] = 4 * i + lc < pw && qc + lq < q1
+                                ? *reinterpret_cast<const float4*>(A + (long)(p0 + 4 * i + lc) * job.ld + p0 + 4 * (qc + lq))
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
             };
             fetch(q0);
-            for (int q = q0; q < q1; ++q) {
-                const int k = p0 + 4 * q;
-                float4 v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] = nv[j];
-                fetch(q + 1);
-                if (k < p0 + QT_NB) {  // the panel's triangle: zeros above the diagonal, ones on it
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int col = 4 * cq + j;
-                        v[j] = make_float4(qt_v(A, job.ld, p0, col, k, v[j].x), qt_v(A, job.ld, p0, col, k + 1, v[j].y),
-                                           qt_v(A, job.ld, p0, col, k + 2, v[j].z),
-                                           qt_v(A, job.ld, p0, col, k + 3, v[j].w));
-                    }
-                }
+            for (int qc = q0; qc < q1; qc += 8) {
+                __syncwarp();
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const float4 x = *reinterpret_cast<const float4*>(X + (size_t)(rq + 4 * i) * ldx + k);
+                    float4 v = nv[i];
+                    const int col = 4 * i + lc, k = p0 + 4 * (qc + lq);
+                    if (k < p0 + QT_NB)  // the panel's triangle: zeros above the diagonal, ones on it
+                        v = make_float4(qt_v(p0, col, k, v.x), qt_v(p0, col, k + 1, v.y), qt_v(p0, col, k + 2, v.z),
+                                        qt_v(p0, col, k + 3, v.w));
+                    Vs[col * 8 + (lq ^ i)] = v;
+                }
+                __syncwarp();
+                fetch(qc + 8);
+                const int nq = min(8, q1 - qc);
+                for (int t = 0; t < nq; ++t) {
+                    const int k = p0 + 4 * (qc + t);
+                    float4 v[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        float a = acc[i][j];
-                        a = fmaf(x.x, v[j].x, a);
-                        a = fmaf(x.y, v[j].y, a);
-                        a = fmaf(x.z, v[j].z, a);
-                        acc[i][j] = fmaf(x.w, v[j].w, a);
+                    for (int j = 0; j < 4; ++j) v[j] = Vs[(4 * cq + j) * 8 + (t ^ cq)];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float4 x = *reinterpret_cast<const float4*>(X + (size_t)(rq + 4 * i) * ldx + k);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            float a = acc[i][j];
+                            a = fmaf(x.x, v[j].x, a);
+                            a = fmaf(x.y, v[j].y, a);
+                            a = fmaf(x.z, v[j].z, a);
+                            acc[i][j] = fmaf(x.w, v[j].w, a);
+                        }
                     }
                 }
             }
+            __syncwarp();
 #pragma unroll
             for (int i = 0; i < 8; ++i)
                 *reinterpret_cast<float4*>(Zp + (size_t)wid * QT_RB * QT_NB + (rq + 4 * i) * QT_NB + 4 * cq) =
@@ -184,8 +195,8 @@ static __global__ void __launch_bounds__(QT_THREADS, 1) k_apply_qt(QtJob<float> 
             if (k < p0 + QT_NB) {  // the panel's triangle
 #pragma unroll
                 for (int j = 0; j < QT_NB; ++j) {
-                    v[j].x = qt_v(A, job.ld, p0, j, k, v[j].x);
-                    v[j].y = qt_v(A, job.ld, p0, j, k + 1, v[j].y);
+                    v[j].x = qt_v(p0, j, k, v[j].x);
+                    v[j].y = qt_v(p0, j, k + 1, v[j].y);
                 }
             }
 #pragma unroll 2
