@@ -107,28 +107,47 @@ __device__ __forceinline__ void adj_below(T (&Z)[NW][4], const AdjOp<T> (&op)[NL
 
 // A dot of float32 blocks in about 48 bits without the FP64 pipe (2 FMAs a clock
 // and SM, which bounded the backward kernel): exact products and TwoSum in
-// float-float; float64 blocks in float64.
-struct AdjDot32 {
+// float-float.  That holds in float32's exponent range only: a product below 2^-149
+// vanishes, one below 2^-102 has no exact error term, one above 2^128 is infinite.
+// A thread loses at most 2^-150 for each of its up to 64 products and error terms, a
+// CTA of 256 threads 2^-136: no more than a float64 sum's rounding beside one dot of
+// at least 2^-82.  seen collects, per layer l, whether there is such a dot (bit l) and
+// whether one is not finite (bit 8 + l); a CTA that misses the one or has the other
+// takes its sums again in float64 (WIDE), as all sums of float64 blocks are.
+template <bool WIDE, int NB>
+__device__ __forceinline__ double adj_dot(const float (&x)[NB], const float (&z)[NB], int l, unsigned& seen) {
+    if constexpr (WIDE) {
+        double s = 0.0;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) s += (double)x[i] * (double)z[i];
+        return s;
+    }
     float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x, float z) {
-        const float p = x * z, e = fmaf(x, z, -p), s = hi + p, bp = s - hi;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const float p = x[i] * z[i], e = fmaf(x[i], z[i], -p), s = hi + p, bp = s - hi;
         lo += ((hi - (s - bp)) + (p - bp)) + e;
         hi = s;
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-struct AdjDot64 {
+    const float t = fabsf(hi + lo);
+    seen |= t >= 0x1p-82f ? 1u << l : 0u;
+    seen |= t <= 0x1p126f ? 0u : 256u << l;
+    return (double)hi + (double)lo;
+}
+template <bool WIDE, int NB>
+__device__ __forceinline__ double adj_dot(const double (&x)[NB], const double (&z)[NB], int, unsigned&) {
     double s = 0.0;
-    __device__ __forceinline__ void add(double x, double z) { s += x * z; }
-    __device__ __forceinline__ double value() const { return s; }
-};
+#pragma unroll
+    for (int i = 0; i < NB; ++i) s += x[i] * z[i];
+    return s;
+}
 
 // part[dl] = X . (M'^dl^T Q) for dl = L .. 0: Z holds Q taken through the layers
 // above; a copy goes through the derivative of layer L and the layers below it,
 // then Z through layer L.  Half of the copy's blocks are zero.
-template <int L, class T, int NW, int NL>
+template <bool WIDE, int L, class T, int NW, int NL>
 __device__ __forceinline__ void adj_derivs(T (&Z)[NW][4], const T (&X)[NW][4], const AdjOp<T> (&op)[NL],
-                                           const AdjOp<T> (&one)[NL], double (&part)[NL]) {
+                                           const AdjOp<T> (&one)[NL], double (&part)[NL], unsigned& seen) {
     T D[NW][4];
 #pragma unroll
     for (int w = 0; w < NW; ++w)
@@ -136,15 +155,16 @@ __device__ __forceinline__ void adj_derivs(T (&Z)[NW][4], const T (&X)[NW][4], c
         for (int n = 0; n < 4; ++n) D[w][n] = Z[w][n];
     adj_layer_bwd<L, true, 0>(D, one[L]);
     adj_below<L, 1 << L>(D, op);
-    std::conditional_t<sizeof(T) == 4, AdjDot32, AdjDot64> d;
+    T xs[2 * NW], ds[2 * NW];  // the entries that are not zero: w without bit L
 #pragma unroll
-    for (int w = 0; w < NW; ++w)
-        if (!(w & (1 << L)))
-#pragma unroll
-            for (int n = 0; n < 4; ++n) d.add(X[w][n], D[w][n]);
-    part[L] = d.value();
+    for (int i = 0; i < 2 * NW; ++i) {
+        const int w = ((i / 4) >> L << (L + 1)) | ((i / 4) & ((1 << L) - 1));
+        xs[i] = X[w][i % 4];
+        ds[i] = D[w][i % 4];
+    }
+    part[L] = adj_dot<WIDE>(xs, ds, L, seen);
     adj_layer_bwd<L, false, 0>(Z, op[L]);
-    if constexpr (L > 0) adj_derivs<L - 1>(Z, X, op, one, part);
+    if constexpr (L > 0) adj_derivs<WIDE, L - 1>(Z, X, op, one, part, seen);
 }
 
 // Y[b][a][n'][w'][bp] = (M_s X)[...] for X[b][a][w][n][bp]; one thread per
@@ -177,59 +197,85 @@ __global__ void __launch_bounds__(256) k_adj_fwd(int Da, int Db, long sb, const 
         for (int w = 0; w < NW; ++w) y[(((long)a * 4 + n) * NW + w) * Db + bp] = Z[w][n];
 }
 
+// One thread's part of the backward kernel: P = M_s^T Q (PUT), and its coefficient
+// gradients.
+template <bool WIDE, bool PUT, class T, int NL>
+__device__ __forceinline__ void adj_bwd_thread(int Db, const T* q, const T* x, T* p, const AdjTerms<T>& tm, int b, int s,
+                                               int a, int bp, double (&part)[NL], unsigned& seen) {
+    constexpr int NW = 1 << NL;
+    T Z[NW][4], Zx[NW][4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int w = 0; w < NW; ++w) Z[w][n] = q[(((long)a * 4 + n) * NW + w) * Db + bp];
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) Zx[w][n] = x[(((long)a * NW + w) * 4 + n) * Db + bp];
+    auto op = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], tm.coef[((long)b * NL + l) * tm.L + s]); };
+    auto one = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], T(1)); };
+    if constexpr (NL == 4) {
+        const AdjOp<T> ops[4] = {op(0), op(1), op(2), op(3)}, ones[4] = {one(0), one(1), one(2), one(3)};
+        adj_derivs<WIDE, 3>(Z, Zx, ops, ones, part, seen);
+    } else {
+        const AdjOp<T> ops[2] = {op(0), op(1)}, ones[2] = {one(0), one(1)};
+        adj_derivs<WIDE, 1>(Z, Zx, ops, ones, part, seen);
+    }
+    if (PUT)
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+#pragma unroll
+            for (int n = 0; n < 4; ++n) p[(((long)a * NW + w) * 4 + n) * Db + bp] = Z[w][n];
+}
+
 // P[b][a][w][n][bp] = (M_s^T Q)[...] for Q[b][a][n'][w'][bp], and
 // g[b][l][s] += sum X . (M'^l^T Q) (the coefficient gradients, reduced per block,
 // one float64 atomic per block and layer).  One thread per (a, bp), blockIdx.y = b.
 template <class T, int NL>
 __global__ void __launch_bounds__(256) k_adj_bwd(int Da, int Db, long sb, const T* Q, T* P, const T* X, double* g,
                                                 AdjTerms<T> tm, int s) {
-    constexpr int NW = 1 << NL;
     __shared__ double red[NL][8];
+    __shared__ unsigned seen_w[8];
     const long per = (long)Da * Db;
     const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
     const bool live = idx < per;
     const int b = blockIdx.y;
     const int a = live ? (int)(idx / Db) : 0, bp = live ? (int)(idx % Db) : 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const T *q = Q + (long)b * sb, *x = X + (long)b * sb;
     double part[NL];
+    auto reduce = [&] {  // the warps' sums to red
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            const double v = warp_sum(part[l]);
+            if (lane == 0) red[l][wid] = v;
+        }
+    };
+    unsigned seen = 0;
 #pragma unroll
     for (int l = 0; l < NL; ++l) part[l] = 0.0;
-    if (live) {
-        const T* q = Q + (long)b * sb;
-        const T* x = X + (long)b * sb;
-        T Z[NW][4], Zx[NW][4];
-#pragma unroll
-        for (int n = 0; n < 4; ++n)
-#pragma unroll
-            for (int w = 0; w < NW; ++w) Z[w][n] = q[(((long)a * 4 + n) * NW + w) * Db + bp];
-#pragma unroll
-        for (int w = 0; w < NW; ++w)
-#pragma unroll
-            for (int n = 0; n < 4; ++n) Zx[w][n] = x[(((long)a * NW + w) * 4 + n) * Db + bp];
-        auto op = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], tm.coef[((long)b * NL + l) * tm.L + s]); };
-        auto one = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], T(1)); };
-        if constexpr (NL == 4) {
-            const AdjOp<T> ops[4] = {op(0), op(1), op(2), op(3)}, ones[4] = {one(0), one(1), one(2), one(3)};
-            adj_derivs<3>(Z, Zx, ops, ones, part);
-        } else {
-            const AdjOp<T> ops[2] = {op(0), op(1)}, ones[2] = {one(0), one(1)};
-            adj_derivs<1>(Z, Zx, ops, ones, part);
-        }
-        T* p = P + (long)b * sb;
-#pragma unroll
-        for (int w = 0; w < NW; ++w)
-#pragma unroll
-            for (int n = 0; n < 4; ++n) p[(((long)a * NW + w) * 4 + n) * Db + bp] = Z[w][n];
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int l = 0; l < NL; ++l) {
-        const double v = warp_sum(part[l]);
-        if (lane == 0) red[l][wid] = v;
+    if (live) adj_bwd_thread<false, true, T, NL>(Db, q, x, P + (long)b * sb, tm, b, s, a, bp, part, seen);
+    reduce();
+    if (sizeof(T) == 4) {
+        seen = __reduce_or_sync(0xffffffffu, seen);
+        if (lane == 0) seen_w[wid] = seen;
     }
     __syncthreads();
+    if constexpr (sizeof(T) == 4) {
+        seen = 0;
+        for (int w = 0; w < nw; ++w) seen |= seen_w[w];
+        if (seen != (1u << NL) - 1) {  // the whole CTA alike
+            __syncthreads();
+#pragma unroll
+            for (int l = 0; l < NL; ++l) part[l] = 0.0;
+            if (live) adj_bwd_thread<true, false, T, NL>(Db, q, x, nullptr, tm, b, s, a, bp, part, seen);
+            reduce();
+            __syncthreads();
+        }
+    }
     if (threadIdx.x < NL) {
         double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
+        for (int w = 0; w < nw; ++w) v += red[threadIdx.x][w];
         atomicAdd(&g[((long)b * NL + threadIdx.x) * tm.L + s], v);
     }
 }
