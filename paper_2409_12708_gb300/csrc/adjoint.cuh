@@ -35,42 +35,57 @@ struct AdjTerms {
     int nl, L;
 };
 
-// A ladder operator's local matrix (c_src, c_sgn) as an index flip: b and b^T of
-// spin up exchange n and n ^ 2, of spin down n and n ^ 1.  Element n' of the
-// result is k[n'] z[n' ^ flip], k = coefficient times sign where the operator has
-// an element and 0 elsewhere, so all register indices are known at compile time
-// (an index from a table puts the blocks into local memory: with it the layer
-// kernels of 1024 terms at L = 10, D = 64 float32 took 35.6 ms, now 5.9 ms).
+// The ladder operators' local matrices (c_src, c_sgn) for an operator known at
+// compile time: two elements, n' = dst <- n = dst ^ flip.  A kernel branches once per
+// layer (the whole CTA alike) to the code of its operator, so that all register
+// indices are constants and only the two elements are multiplied: an entry that the
+// operator does not reach is left alone, also by an infinity (a coefficient of zero
+// would make it NaN).  Layer kernels of all terms at L = 8, N = 8, D = 64 against four
+// products of which two have a zero coefficient: float64 4.51 -> 3.13 ms, float32
+// (bound elsewhere) within 2 %.  Indices from a table would put the blocks into local
+// memory: 35.6 against 5.9 ms for 1024 terms at L = 10, D = 64, float32.
+__device__ __forceinline__ constexpr int adj_par(int n) { return n == 0 || n == 3 ? 1 : -1; }  // c_par
+template <int O>  // O = sigma + 2 dagger
+struct AdjMat {
+    static constexpr int flip = O & 1 ? 1 : 2;
+    // output n' has an element (annihilation: the mode is empty in n'), its sign
+    static __device__ __forceinline__ constexpr bool has(int np) { return ((np & flip) != 0) == (O >= 2); }
+    static __device__ __forceinline__ constexpr int sgn(int np) { return (O & 1) && (np & 2) ? -1 : 1; }
+};
+template <class F>
+__device__ __forceinline__ void adj_by_op(int o, F f) {
+    switch (o) {
+        case 0: f(AdjMat<0>{}); break;
+        case 1: f(AdjMat<1>{}); break;
+        case 2: f(AdjMat<2>{}); break;
+        default: f(AdjMat<3>{}); break;
+    }
+}
 template <class T>
 struct AdjOp {
-    bool up;   // flips bit 1 of n, else bit 0
-    T k[4];
-    __device__ __forceinline__ AdjOp(int o, T c) : up((o & 1) == 0) {
-#pragma unroll
-        for (int n = 0; n < 4; ++n) k[n] = c * T(c_sgn[o][n]);
-    }
-    __device__ __forceinline__ T flip(const T (&z)[4], int n) const { return up ? z[n ^ 2] : z[n ^ 1]; }
+    int o;
+    T c;
 };
-__device__ __forceinline__ constexpr int adj_par(int n) { return n == 0 || n == 3 ? 1 : -1; }  // c_par
 
 // Layer l applied to the block Z[w][n] (2^NL x 4) at site s (input side bit l = a,
 // output side bit l = b): Z'[b=0][n'] = par[n'] Z[a=0][n'],
 // Z'[b=1][n'] = c sgn[n'] Z[a=0][src[n']] + Z[a=1][n'].
 template <int L, class T, int NW>
 __device__ __forceinline__ void adj_layer_fwd(T (&Z)[NW][4], const AdjOp<T>& op) {
+    adj_by_op(op.o, [&](auto mat) {
+        using M = decltype(mat);
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        if (w & (1 << L)) continue;
-        const int w1 = w | (1 << L);
-        T z0[4];
+        for (int w = 0; w < NW; ++w) {
+            if (w & (1 << L)) continue;
+            const int w1 = w | (1 << L);
 #pragma unroll
-        for (int n = 0; n < 4; ++n) z0[n] = Z[w][n];
+            for (int n = 0; n < 4; ++n)
+                if (M::has(n)) Z[w1][n] += (M::sgn(n) < 0 ? -op.c : op.c) * Z[w][n ^ M::flip];
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            Z[w][n] = T(adj_par(n)) * z0[n];
-            Z[w1][n] += op.k[n] * op.flip(z0, n);
+            for (int n = 0; n < 4; ++n)
+                if (adj_par(n) < 0) Z[w][n] = -Z[w][n];
         }
-    }
+    });
 }
 
 // Transposed layer l on the output-side block Z[w'][n'] -> input side:
@@ -80,22 +95,25 @@ __device__ __forceinline__ void adj_layer_fwd(T (&Z)[NW][4], const AdjOp<T>& op)
 // Z'[a=1] = 0.  ZERO: bits of w whose blocks are zero (below a derivative) and skipped.
 template <int L, bool DERIV, int ZERO, class T, int NW>
 __device__ __forceinline__ void adj_layer_bwd(T (&Z)[NW][4], const AdjOp<T>& op) {
+    adj_by_op(op.o, [&](auto mat) {
+        using M = decltype(mat);
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        if ((w & (1 << L)) || (w & ZERO)) continue;
-        const int w1 = w | (1 << L);
-        T t[4];
+        for (int w = 0; w < NW; ++w) {
+            if ((w & (1 << L)) || (w & ZERO)) continue;
+            const int w1 = w | (1 << L);
 #pragma unroll
-        for (int n = 0; n < 4; ++n) t[n] = op.k[n];
+            for (int n = 0; n < 4; ++n) {
+                const int np = n ^ M::flip;
+                const T z1 = M::sgn(np) < 0 ? -Z[w1][np] : Z[w1][np];
+                if (DERIV) Z[w][n] = M::has(np) ? z1 : T(0);
+                else if (M::has(np)) Z[w][n] = op.c * z1 + (adj_par(n) < 0 ? -Z[w][n] : Z[w][n]);
+                else if (adj_par(n) < 0) Z[w][n] = -Z[w][n];
+            }
+            if (DERIV)
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            const T kk = op.up ? t[n ^ 2] : t[n ^ 1], z1 = op.flip(Z[w1], n);
-            Z[w][n] = DERIV ? kk * z1 : T(adj_par(n)) * Z[w][n] + kk * z1;
+                for (int n = 0; n < 4; ++n) Z[w1][n] = T(0);
         }
-        if (DERIV)
-#pragma unroll
-            for (int n = 0; n < 4; ++n) Z[w1][n] = T(0);
-    }
+    });
 }
 template <int L, int ZERO, class T, int NW, int NL>
 __device__ __forceinline__ void adj_below(T (&Z)[NW][4], const AdjOp<T> (&op)[NL]) {  // layers L-1 .. 0
@@ -147,13 +165,13 @@ __device__ __forceinline__ double adj_dot(const double (&x)[NB], const double (&
 // then Z through layer L.  Half of the copy's blocks are zero.
 template <bool WIDE, int L, class T, int NW, int NL>
 __device__ __forceinline__ void adj_derivs(T (&Z)[NW][4], const T (&X)[NW][4], const AdjOp<T> (&op)[NL],
-                                           const AdjOp<T> (&one)[NL], double (&part)[NL], unsigned& seen) {
+                                           double (&part)[NL], unsigned& seen) {
     T D[NW][4];
 #pragma unroll
     for (int w = 0; w < NW; ++w)
 #pragma unroll
         for (int n = 0; n < 4; ++n) D[w][n] = Z[w][n];
-    adj_layer_bwd<L, true, 0>(D, one[L]);
+    adj_layer_bwd<L, true, 0>(D, op[L]);
     adj_below<L, 1 << L>(D, op);
     T xs[2 * NW], ds[2 * NW];  // the entries that are not zero: w without bit L
 #pragma unroll
@@ -164,7 +182,7 @@ __device__ __forceinline__ void adj_derivs(T (&Z)[NW][4], const T (&X)[NW][4], c
     }
     part[L] = adj_dot<WIDE>(xs, ds, L, seen);
     adj_layer_bwd<L, false, 0>(Z, op[L]);
-    if constexpr (L > 0) adj_derivs<WIDE, L - 1>(Z, X, op, one, part, seen);
+    if constexpr (L > 0) adj_derivs<WIDE, L - 1>(Z, X, op, part, seen);
 }
 
 // Y[b][a][n'][w'][bp] = (M_s X)[...] for X[b][a][w][n][bp]; one thread per
@@ -183,7 +201,7 @@ __global__ void __launch_bounds__(256) k_adj_fwd(int Da, int Db, long sb, const 
     for (int w = 0; w < NW; ++w)
 #pragma unroll
         for (int n = 0; n < 4; ++n) Z[w][n] = x[(((long)a * NW + w) * 4 + n) * Db + bp];
-    auto op = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], tm.coef[((long)b * NL + l) * tm.L + s]); };
+    auto op = [&](int l) { return AdjOp<T>{tm.op[b * NL + l], tm.coef[((long)b * NL + l) * tm.L + s]}; };
     adj_layer_fwd<0>(Z, op(0));
     adj_layer_fwd<1>(Z, op(1));
     if constexpr (NL == 4) {
@@ -212,14 +230,13 @@ __device__ __forceinline__ void adj_bwd_thread(int Db, const T* q, const T* x, T
     for (int w = 0; w < NW; ++w)
 #pragma unroll
         for (int n = 0; n < 4; ++n) Zx[w][n] = x[(((long)a * NW + w) * 4 + n) * Db + bp];
-    auto op = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], tm.coef[((long)b * NL + l) * tm.L + s]); };
-    auto one = [&](int l) { return AdjOp<T>(tm.op[b * NL + l], T(1)); };
+    auto op = [&](int l) { return AdjOp<T>{tm.op[b * NL + l], tm.coef[((long)b * NL + l) * tm.L + s]}; };
     if constexpr (NL == 4) {
-        const AdjOp<T> ops[4] = {op(0), op(1), op(2), op(3)}, ones[4] = {one(0), one(1), one(2), one(3)};
-        adj_derivs<WIDE, 3>(Z, Zx, ops, ones, part, seen);
+        const AdjOp<T> ops[4] = {op(0), op(1), op(2), op(3)};
+        adj_derivs<WIDE, 3>(Z, Zx, ops, part, seen);
     } else {
-        const AdjOp<T> ops[2] = {op(0), op(1)}, ones[2] = {one(0), one(1)};
-        adj_derivs<WIDE, 1>(Z, Zx, ops, ones, part, seen);
+        const AdjOp<T> ops[2] = {op(0), op(1)};
+        adj_derivs<WIDE, 1>(Z, Zx, ops, part, seen);
     }
     if (PUT)
 #pragma unroll
