@@ -627,25 +627,78 @@ __device__ __forceinline__ void qr_t_matrix(const QrCtx<T, NB, S, NQ>& x, int pw
     __syncthreads();
 }
 
+// The metric of columns which (bits) of this group's quad, measured: their squared
+// norms from row j down.
+template <int NA, class T, int NB, int S, int NQ>
+__device__ __forceinline__ void qr_remeasure(const QrCtx<T, NB, S, NQ>& x, const QrQuad<T, NQ>& y, int j, unsigned which,
+                                             real_t<T>* met) {
+    constexpr int V = QrVec<T>::V;
+    using RT = real_t<T>;
+    if (which == 0) return;  // the group's warps alike
+    RT s2[QR_NC];
+#pragma unroll
+    for (int c = 0; c < QR_NC; ++c) {
+        s2[c] = RT(0);
+#pragma unroll
+        for (int q = 0; q < NA; ++q)
+#pragma unroll
+            for (int e = 0; e < V; ++e)  // rows above j lie in the first chunk
+                if (q > 0 || x.row(0) + e >= j) s2[c] += tabs2(y[c][q][e]);
+    }
+    RT t = qr_reduce_scatter<QR_NC>(s2);
+    const int c = x.lane >> 3;
+    if constexpr (S > 1) {
+        RT* pd = reinterpret_cast<RT*>(x.pd + x.grp * S * QR_NC);
+        if ((x.lane & 7) == 0) pd[x.h * QR_NC + c] = t;
+        x.sync();
+        t = RT(0);
+#pragma unroll 1
+        for (int hh = 0; hh < S; ++hh) t += pd[hh * QR_NC + c];
+    }
+    if (x.h == 0 && (x.lane & 7) == 0 && ((which >> c) & 1u)) met[x.grp * QR_NC + c] = t;
+}
+
+// A metric is measured again once less than sqrt(eps) of the value last measured is
+// left (the rule of Drmac and Bujanovic for pivoted QR): the differences then have
+// lost half of their digits.
+template <class RT>
+constexpr RT QR_STALE = sizeof(RT) == 4 ? RT(2.4414062e-4) : RT(1.0536712e-8);
+
 // Householder factorisation of the panel: group g holds columns 4 g .. 4 g + 3
 // of the pw panel columns in y (R rows).  Per step: the owner forms the
 // reflector (qr_reflect), one CTA barrier, then every group takes the dots of
 // v with its four columns and updates those not yet done; the dots with
-// finished columns are the entries of G = V^H V, which give T at the end.  Pivoting (met != null): step j
-// takes the remaining column with the largest metric (its squared norm at the
-// start of the panel, reduced by the squares of the R entries found since);
-// stp[c] is the step at which this group's column c was taken.
+// finished columns are the entries of G = V^H V, which give T at the end.  Pivoting
+// (met != null): step j takes the remaining column with the largest metric, its
+// squared norm: at the start of the panel a plain sum in the storage type, reduced by
+// the squares of the R entries found since, and measured again from the quad's
+// registers where that has cancelled (otherwise graded and rank-deficient panels are
+// taken in the order of rounding noise, and their factors cost the Jacobi sweeps).
+// float64 metrics are compared by their upper 32 bits (1e-6).  stp[c] is the step at
+// which this group's column c was taken.
 template <int NA, bool PIV, class T, int NB, int S, int NQ>
 __device__ __forceinline__ void qr_panel(const QrCtx<T, NB, S, NQ>& x, QrQuad<T, NQ>& y, int pw, bool want_t,
                                          real_t<T>* met, int (&stp)[QR_NC]) {
     constexpr int V = QrVec<T>::V;
 #pragma unroll
     for (int c = 0; c < QR_NC; ++c) stp[c] = NB;
+    real_t<T> ref = real_t<T>(0);  // lane's column: its metric when last measured
 #pragma unroll 1
     for (int j = 0; j < pw; ++j) {
         int k = j;
         if (PIV) {
-            const int key = x.lane < pw ? (met[x.lane] == real_t<T>(-2) ? -2 : qr_metric_key(met[x.lane])) : -2;
+            real_t<T> mv = x.lane < pw ? met[x.lane] : real_t<T>(-2);
+            if (j == 0) ref = mv;
+            const bool stale = mv >= real_t<T>(0) && mv < QR_STALE<real_t<T>> * ref;
+            const unsigned which = __ballot_sync(0xffffffffu, stale);
+            if (which) {  // the whole CTA alike: every warp reads the same metrics
+                __syncthreads();
+                qr_remeasure<NA>(x, y, j, (which >> (x.grp * QR_NC)) & 15u, met);
+                __syncthreads();
+                if (x.lane < pw) mv = met[x.lane];
+                if (stale) ref = mv;
+            }
+            const int key = mv == real_t<T>(-2) ? -2 : qr_metric_key(mv);
             const int best = __reduce_max_sync(0xffffffffu, key);
             k = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
         }
