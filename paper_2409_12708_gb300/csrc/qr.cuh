@@ -79,8 +79,9 @@ struct QrShape {
 // serial chain) overlaps the other's update: 304 pivoted 512 x 256 float32
 // matrices take 1.07 ms that way and 1.57 ms with two warps per quad, and one
 // matrix alone 0.75 against 0.77 ms.
-constexpr QrShape QR_SHAPES[] = {{32, 1, 2}, {32, 1, 4}, {32, 2, 4}, {16, 4, 4}, {8, 8, 4}, {4, 16, 4}};
-constexpr int QR_NSHAPES = 6;
+constexpr QrShape QR_SHAPES[] = {{32, 1, 2}, {32, 1, 4}, {32, 2, 4}, {16, 4, 4}, {8, 8, 4}, {4, 16, 4},
+                                 {16, 2, 2}, {16, 2, 4}};
+constexpr int QR_NSHAPES = 8;
 
 // Chunks per lane and column that a panel of R rows works on: all or half of
 // them, so that the inner loops have no branch per chunk.
@@ -103,10 +104,22 @@ __host__ inline size_t qr_smem_bytes(const QrShape& sh, int m, int n, bool pivot
     return elems * sizeof(T) + 3 * warps * 16 + ((piv + 15) & ~(size_t)15);
 }
 
+// Pivoted matrices of 8- and 16-byte scalars with n >= 128 take panels of 16 columns:
+// columns are sorted once per panel, so a narrower one pivots better and saves the
+// Jacobi sweeps, which cost most where rows are long.  float64 factors with n >= 128
+// of 16 terms at L = 16, D = 128: 3296 sweeps against 3411, 7.12 against 7.52 s, the QR
+// itself 787 against 790 ms.  Below, 16 columns cost as much or more: 11344 against
+// 11199 sweeps at L = 6, D = 16 float64, 344.6 against 341.6 ms for H|psi> at L = 6,
+// D = 32 complex128.
+template <class T>
+constexpr bool qr_narrow(bool pivot) { return pivot && sizeof(T) >= 8; }
+
 // The shape for m rows (negative: none).
 template <class T>
 __host__ inline int qr_shape(int m, int n, bool pivot, size_t smem_max) {
-    for (int i = 0; i < QR_NSHAPES; ++i) {
+    const bool narrow = qr_narrow<T>(pivot) && n >= 128;
+    for (int i : {narrow ? 6 : 0, narrow ? 7 : 1, 2, 3, 4, 5}) {
+        if (narrow && i == 2) continue;
         if (QR_SHAPES[i].units() * 32 * QrVec<T>::V < m) continue;
         if (qr_smem_bytes<T>(QR_SHAPES[i], m, n, pivot) <= smem_max) return i;
     }
@@ -998,13 +1011,17 @@ __global__ void __launch_bounds__(32 * S * NB / QR_NC, S == 1 ? 2 : 1) k_qr(QRJo
 // f(kernel) for shape i of QR_SHAPES
 template <class T, bool PIV, class F>
 inline void qr_dispatch(int shape, F&& f) {
+    if constexpr (qr_narrow<T>(PIV)) {
+        if (shape == 6) return f(k_qr<T, 16, 2, 2, PIV>);
+        if (shape == 7) return f(k_qr<T, 16, 2, 4, PIV>);
+    }
     switch (shape) {
         case 0: return f(k_qr<T, 32, 1, 2, PIV>);
         case 1: return f(k_qr<T, 32, 1, 4, PIV>);
         case 2: return f(k_qr<T, 32, 2, 4, PIV>);
         case 3: return f(k_qr<T, 16, 4, 4, PIV>);
         case 4: return f(k_qr<T, 8, 8, 4, PIV>);
-        default: return f(k_qr<T, 4, 16, 4, PIV>);
+        case 5: return f(k_qr<T, 4, 16, 4, PIV>);
     }
 }
 

@@ -18,7 +18,7 @@ from kernel_harness import compile_kernels, pointer  # noqa: E402
 
 # (scalar, panel width, warps per quad, chunks): one and several warps per quad
 SHAPES = {"f32_1": ("float", 32, 1, 2), "f32_2": ("float", 32, 2, 4), "f32_8": ("float", 8, 8, 4),
-          "f64_1": ("double", 32, 1, 2), "c64_1": ("cplx<float>", 32, 1, 2)}
+          "f64_1": ("double", 32, 1, 2), "f64_2": ("double", 16, 2, 4), "f64_h": ("double", 16, 2, 2), "c64_1": ("cplx<float>", 32, 1, 2)}
 SOURCE = r"""
 #include "qr.cuh"
 using namespace thc;
@@ -65,7 +65,7 @@ def spectrum(kind, n, scalar):
 
 @pytest.mark.parametrize("kind", ["graded", "deficient", "step", "mild"])
 @pytest.mark.parametrize("shape,m,n", [("f32_1", 64, 32), ("f32_1", 256, 47), ("f32_2", 512, 40), ("f32_8", 400, 24),
-                                       ("f64_1", 128, 40), ("c64_1", 128, 32)])
+                                       ("f64_1", 128, 40), ("f64_2", 500, 70), ("f64_h", 256, 52), ("c64_1", 128, 32)])
 def test_each_step_takes_the_largest_remaining_column(lib, kind, shape, m, n):
     scalar, nb, B = shape[:3], SHAPES[shape][1], 6
     rng = np.random.default_rng(m + n)
