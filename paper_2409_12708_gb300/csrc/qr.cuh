@@ -597,9 +597,19 @@ __device__ __forceinline__ void qr_reflect(const QrCtx<T, NB, S, NQ>& x, T (&y)[
     if (x.h == 0 && x.lane == 0) x.Tm[j * x.LDT + j] = tau;
 }
 
-// Order of a non-negative metric as an integer (NaN and negative values last).
-__device__ __forceinline__ int qr_metric_key(float v) { return v >= 0.f ? __float_as_int(v) : -1; }
-__device__ __forceinline__ int qr_metric_key(double v) { return v >= 0.0 ? __double2hiint(v) : -1; }
+// Order of a non-negative metric as an integer: float32's bits, float64's upper 32 (so
+// metrics within 1e-6 are alike); NaN and negative values -1, a taken column (-2) -2.
+// On integers throughout: a float64 comparison would hold the FP64 pipe for 16 clocks
+// a warp in every step of the panel.
+constexpr int QR_TAKEN = -2;
+__device__ __forceinline__ int qr_metric_key(float v) {
+    const int i = __float_as_int(v);
+    return i == (int)0xc0000000u ? QR_TAKEN : i < 0 || i > 0x7f800000 ? -1 : i;
+}
+__device__ __forceinline__ int qr_metric_key(double v) {
+    const int i = __double2hiint(v);
+    return i == (int)0xc0000000u ? QR_TAKEN : i < 0 || i > 0x7ff00000 ? -1 : i;
+}
 
 // T of the compact WY form from tau on its diagonal and G = V^H V: with the
 // columns in two halves, T = [T1, -T1 G12 T2; 0, T2], so blocks of 1, 2, 4, ...
@@ -671,11 +681,11 @@ __device__ __forceinline__ void qr_remeasure(const QrCtx<T, NB, S, NQ>& x, const
     if (x.h == 0 && (x.lane & 7) == 0 && ((which >> c) & 1u)) met[x.grp * QR_NC + c] = t;
 }
 
-// A metric is measured again once less than sqrt(eps) of the value last measured is
-// left (the rule of Drmac and Bujanovic for pivoted QR): the differences then have
-// lost half of their digits.
+// A metric is measured again once less than sqrt(eps) (2^-12, 2^-27) of the value last
+// measured is left (the rule of Drmac and Bujanovic for pivoted QR): the differences
+// then have lost half of their digits.  As a distance of metric keys.
 template <class RT>
-constexpr RT QR_STALE = sizeof(RT) == 4 ? RT(2.4414062e-4) : RT(1.0536712e-8);
+constexpr int QR_STALE = sizeof(RT) == 4 ? 12 << 23 : 27 << 20;
 
 // Householder factorisation of the panel: group g holds columns 4 g .. 4 g + 3
 // of the pw panel columns in y (R rows).  Per step: the owner forms the
@@ -695,23 +705,21 @@ __device__ __forceinline__ void qr_panel(const QrCtx<T, NB, S, NQ>& x, QrQuad<T,
     constexpr int V = QrVec<T>::V;
 #pragma unroll
     for (int c = 0; c < QR_NC; ++c) stp[c] = NB;
-    real_t<T> ref = real_t<T>(0);  // lane's column: its metric when last measured
+    int ref = 0;  // lane's column: its metric's key when last measured
 #pragma unroll 1
     for (int j = 0; j < pw; ++j) {
         int k = j;
         if (PIV) {
-            real_t<T> mv = x.lane < pw ? met[x.lane] : real_t<T>(-2);
-            if (j == 0) ref = mv;
-            const bool stale = mv >= real_t<T>(0) && mv < QR_STALE<real_t<T>> * ref;
+            int key = x.lane < pw ? qr_metric_key(met[x.lane]) : QR_TAKEN;
+            if (j == 0) ref = key;
+            const bool stale = key >= 0 && key < ref - QR_STALE<real_t<T>>;
             const unsigned which = __ballot_sync(0xffffffffu, stale);
             if (which) {  // the whole CTA alike: every warp reads the same metrics
                 __syncthreads();
                 qr_remeasure<NA>(x, y, j, (which >> (x.grp * QR_NC)) & 15u, met);
                 __syncthreads();
-                if (x.lane < pw) mv = met[x.lane];
-                if (stale) ref = mv;
+                if (stale) ref = key = qr_metric_key(met[x.lane]);
             }
-            const int key = mv == real_t<T>(-2) ? -2 : qr_metric_key(mv);
             const int best = __reduce_max_sync(0xffffffffu, key);
             k = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
         }
@@ -750,7 +758,7 @@ __device__ __forceinline__ void qr_panel(const QrCtx<T, NB, S, NQ>& x, QrQuad<T,
             }
         }
         __syncthreads();
-        if (PIV && kc >= 0 && x.h == 0 && x.lane == 0) met[k] = real_t<T>(-2);
+        if (PIV && kc >= 0 && x.h == 0 && x.lane == 0) met[k] = real_t<T>(QR_TAKEN);
         // a group whose columns are all done has only its entries of G left to give
         const bool live = max(max(stp[0], stp[1]), max(stp[2], stp[3])) == NB || want_t;
         if (x.grp * QR_NC < pw && live) {
