@@ -845,7 +845,27 @@ __global__ void __launch_bounds__(32 * S * NB / QR_NC, S == 1 ? 2 : 1) k_qr(QRJo
     QrCtx<T, NB, S, NQ> x;
     x.ldp = qr_ldp<T>(m, S, NQ);
     x.grp = wid / S;
-    x.h = wid % S;
+    // the warps of a quad by rank h; where chunks past the matrix are left out (below), the
+    // last rank's empty first, and a warp's place in the CTA fixes its scheduler: ranks are
+    // turned from quad to quad
+    x.h = (wid + (sizeof(RT) < 8 ? 0 : S >= 4 ? x.grp : x.grp / 2)) % S;
+    // Y's update.  The FP64 pipe bounds 64-bit types, so each warp takes only the chunks
+    // that hold rows (at 1024 x 256, 12 to 16 of the quad's 16): 120 LQ launches of 16 terms
+    // at L = 16, D = 128 float64 2717 -> 2597 ms, the pivoted QRs 788 -> 739 ms.  (A branch
+    // per chunk in the loops gained nothing: 2755 ms.)  32-bit types keep two versions.
+    auto update = [&](QrQuad<T, NQ>& yy, int pw, int R, bool adj) {
+        if constexpr (sizeof(RT) == 8 && NQ == 4) {
+            const int act = (ceil_div(R, 32 * V) - x.h + S - 1) / S;
+            if (act >= 4) qr_apply_quad<4>(x, yy, pw, adj);
+            else if (act == 3) qr_apply_quad<3>(x, yy, pw, adj);
+            else if (act == 2) qr_apply_quad<2>(x, yy, pw, adj);
+            else qr_apply_quad<1>(x, yy, pw, adj);
+        } else if (qr_active(R, V, S, NQ) == NQ) {
+            qr_apply_quad<NQ>(x, yy, pw, adj);
+        } else {
+            qr_apply_quad<NQ / 2>(x, yy, pw, adj);
+        }
+    };
     x.lane = lane;
     x.pn = smem_raw;
     x.pa = smem_raw + 2 * x.WARPS * 16;
@@ -930,8 +950,7 @@ __global__ void __launch_bounds__(32 * S * NB / QR_NC, S == 1 ? 2 : 1) k_qr(QRJo
 #pragma unroll
             for (int c = 0; c < QR_NC; ++c) col[c] = c0 + c < n ? A + (long)phys(c0 + c) * ld + p0 : nullptr;
             qr_load<T, NB, S, NQ>(x, y, col, R);
-            if (full) qr_apply_quad<NQ>(x, y, pw, true);
-            else qr_apply_quad<NQ / 2>(x, y, pw, true);
+            update(y, pw, R, true);
             qr_store<T, NB, S, NQ>(x, y, col, R);
             if (PIV) {  // their norms below row p0 + pw, for the next panel
                 RT s2[QR_NC];
@@ -983,7 +1002,6 @@ __global__ void __launch_bounds__(32 * S * NB / QR_NC, S == 1 ? 2 : 1) k_qr(QRJo
             const int p0 = pi * nb;
             const int pw = min(nb, kk - p0);
             const int R = m - p0;
-            const bool full = qr_active(R, V, S, NQ) == NQ;
             for (int o = tid; o < pw * x.ldp; o += nt) {
                 const int i = o / x.ldp, r = o % x.ldp;
                 x.P[o] = r < i || r >= R ? tzero<T>() : (r == i ? tone<T>() : A[(long)(p0 + i) * ld + p0 + r]);
@@ -1006,8 +1024,7 @@ __global__ void __launch_bounds__(32 * S * NB / QR_NC, S == 1 ? 2 : 1) k_qr(QRJo
                 } else {
                     qr_load<T, NB, S, NQ>(x, y, col, R);
                 }
-                if (full) qr_apply_quad<NQ>(x, y, pw, false);
-                else qr_apply_quad<NQ / 2>(x, y, pw, false);
+                update(y, pw, R, false);
                 qr_store<T, NB, S, NQ>(x, y, col, R);
             }
             for (int i = tid; i < pw * p0; i += nt) A[(long)(p0 + i / p0) * ld + i % p0] = tzero<T>();
