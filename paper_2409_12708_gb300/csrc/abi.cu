@@ -151,7 +151,7 @@ thc_status thc_apply_H_batched(int n, const thc_hamiltonian* const* H, const thc
         // the instances' terms in flight share the device: split the default
         thc_opts o = *opts;
         if (o.batch <= 0) {
-            int dev = 0, sms = 152;
+            int dev = 0, sms = thc::GB300_SMS;
             THC_CUDA(cudaGetDevice(&dev));
             THC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
             o.batch = std::max(32, 4 * sms / n);

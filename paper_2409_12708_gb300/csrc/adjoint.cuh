@@ -18,8 +18,9 @@
 //       tensor replaced by dW/dc_s = [[0, b], [0, 0]];
 //   d value / d psi_s = E_s^T (M_s^T Q_s).
 // Each site is four batched GEMMs (the library's tiled GEMM) and two
-// register-resident kernels that apply the layers (forward, or transposed
-// with the coefficient gradients).  Real MPS only.
+// kernels that apply the layers in registers (forward, or transposed with the
+// coefficient gradients; the transposed one of four float64 layers holds three blocks of
+// 64 entries and spills 316 bytes of them).  Real MPS only.
 #pragma once
 
 #include "common.cuh"

@@ -64,6 +64,8 @@ __device__ __forceinline__ double block_max(double v, double* red) {
     return r;
 }
 
+constexpr int GB300_SMS = 152;  // for choices made without a device query
+
 __host__ __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // square root and sign transfer in the storage precision (no silent promotion)

@@ -209,7 +209,7 @@ struct Plan {
     std::vector<int> out;        // bonds after the SVD sweep
     std::vector<long> woff;      // slot s: X_s [e[s] x 4 k[s+1]]
     long wsize = 0;
-    long maxL = 0, maxC = 0, maxZ = 0, maxV = 0, maxTw = 0, maxKout = 0, maxQRm = 0;
+    long maxL = 0, maxC = 0, maxZ = 0, maxV = 0, maxTw = 0, maxKout = 0;
     int maxP = 0, maxN = 0;
 };
 
@@ -250,7 +250,6 @@ inline Plan make_plan(int mode, const std::vector<int>& inA, const std::vector<i
         if (s >= 1) {
             const int nb = QR_SHAPES[qr_params<T>(m, n, false)].nb;
             P.maxTw = std::max(P.maxTw, (long)ceil_div(std::min(m, n), nb) * nb * nb);
-            P.maxQRm = std::max<long>(P.maxQRm, m);
         }
     }
     for (int s = 0; s < L - 1; ++s) {
@@ -262,10 +261,7 @@ inline Plan make_plan(int mode, const std::vector<int>& inA, const std::vector<i
         P.maxKout = std::max<long>(P.maxKout, P.out[s + 1]);
         P.maxP = std::max(P.maxP, p);
         P.maxN = std::max(P.maxN, n);
-        if (m >= n) {
-            qr_params<T>(m, n, true);  // refuses what no launch shape covers
-            P.maxQRm = std::max<long>(P.maxQRm, m);
-        }
+        if (m >= n) qr_params<T>(m, n, true);  // refuses what no launch shape covers
     }
     return P;
 }

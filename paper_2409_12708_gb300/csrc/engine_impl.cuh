@@ -39,7 +39,7 @@ struct Engine {
     Alloc al;
     int* dflag = nullptr;  // device status word
     double* ddbg = nullptr;  // device diagnostics of a non-converged Jacobi ([4])
-    int sms = 152;
+    int sms = GB300_SMS;
     int smem_optin = 227 * 1024;  // largest dynamic shared memory a block may opt in to
 
     Engine(cudaStream_t s, const thc_allocator* a) : st(s) {

@@ -85,7 +85,8 @@ struct WalkM<LA, std::enable_if_t<LA::walk_m>> : std::true_type {};
 // every k step at 128 x 128 reads its operands with four 16-byte shared-memory
 // loads for 64 multiply-adds, done on packed pairs of columns (32 instructions).
 // The next BK-slice of the operands is loaded into registers while this one is
-// multiplied, and two CTAs share an SM (slices of 8: with 16 the prefetch spills).
+// multiplied, and two CTAs share an SM, which caps a thread at 128 registers: at
+// 128 x 128 with slices of 8 some loaders spill 16 to 56 bytes, with 16 all do, to 232.
 // Bound by the FMA pipe and by the functors' index arithmetic.  Measured: expand +
 // absorb of 608 terms at L = 16, D = 128 83.5 -> 61.6 ms; the products of a gradient
 // at L = 10, N = 30, D = 64 (bond 64: the 64-wide tiles) 41.9 -> 26.9 ms against
@@ -266,7 +267,7 @@ inline cudaError_t launch_gemm(int batch, int M, int N, int K, const LA& la, con
     using Tile32 = std::integral_constant<int, 32>;
     if constexpr (sizeof(real_t<Acc>) == 8) {
         const long tiles = (long)batch * ceil_div(M, 32) * ceil_div(N, 32);
-        return M > 16 && N > 16 && tiles >= 2 * 152 ? small(Tile32{}) : small(Tile16{});
+        return M > 16 && N > 16 && tiles >= 2 * GB300_SMS ? small(Tile32{}) : small(Tile16{});
     } else {
         if (M <= 16 && N <= 16) return small(Tile16{});
         if (M <= 32 || N <= 32) return small(Tile32{});

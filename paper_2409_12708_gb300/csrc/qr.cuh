@@ -11,21 +11,28 @@
 //
 // Work split.  Columns are held in registers, four ("a quad") per group of S
 // warps: lane l of warp h of the group holds 16-byte chunks of rows
-// ((q S + h) 32 + l) VEC, q < 4, of the four columns (64 registers).  The panel
-// of nb = 64 / S columns is factored by all groups at once, each on its own
-// quad; the finished reflectors V go to shared memory, and every trailing quad
+// ((q S + h) 32 + l) VEC, q < NQ, of the four columns (16 NQ 32-bit registers).  The
+// panel of nb columns (QR_SHAPES) is factored by all nb / 4 groups at once, each on
+// its own quad; the finished reflectors V go to shared memory, and every trailing quad
 // then is loaded into registers once, updated (W = V^H Y, W <- T^H W,
 // Y -= V W) and stored once.  A group needs only its own warps for that (a
 // named barrier), so the groups run free of each other between panels and hide
 // one another's load latency; the CTA-wide barriers are one per panel column
 // (two when pivoting).  A 16-byte load of V from shared memory feeds four
 // columns, so the FMA pipe and the shared-memory pipe are about evenly loaded.
-// What bounds it: the panel columns' serial chain (norm, scalars, barrier, dots,
-// update: about 1500 cycles a column), then the FMA pipe of the updates (36 %
-// busy over the launch).  Measured (GB300, float32): 304 matrices of 1024 x 256
-// in 2.04 ms, one alone in 0.97 ms (4.55 and 2.14 ms with groups of 16 columns
-// updated straight from global memory behind four CTA barriers each); 304 of
-// 512 x 256 pivoted in 1.07 ms, one in 0.75 ms (3.43 and 1.69 ms).
+// What bounds it.  float32: about half the panel columns' serial chain (norm, scalars,
+// barrier, dots, update), half the updates.  Shares of a warp's time by the clock, one
+// 1024 x 256 matrix (beside 303 others within two points the same): panel columns 44 %
+// (3160 cycles a column), W 23 %, Y -= V W 15 %, T^H W with its barriers 5 %, T 4 %, loads
+// of quads and panels 4 %, stores and outputs 4 %, waiting at the end of a panel 1 %;
+// 512 x 256 pivoted: 50 (3400 cycles), 16, 10, 6, 5, 7, 6, 1.  Neither pipe is full: issue
+// 0.38 a scheduler (pivoted 0.48), FMA-pipe instructions 21 (24) % of peak, most of them packed
+// pairs, warps waiting at barriers first, then for the arithmetic itself.  float64: the
+// FP64 pipe (2 FMAs a clock and SM): W 42 %, Y -= V W 33 %, panel columns 15 %.
+// Measured (GB300, float32): 304 matrices of 1024 x 256 in 2.04 ms, one alone in
+// 0.97 ms (4.55 and 2.14 ms with groups of 16 columns updated straight from global
+// memory behind four CTA barriers each); 304 of 512 x 256 pivoted in 1.06 ms, one in
+// 0.75 ms (3.43 and 1.69 ms).
 //
 // Modes (after the factorisation):
 //   QR_L_AND_Q : writes L = R^T (n x kk, row-major) and overwrites the first kk
@@ -156,7 +163,6 @@ struct SqAcc<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double x) { s += x * x; }
     __device__ __forceinline__ void merge(const SqAcc& o) { s += o.s; }
-    __device__ __forceinline__ double warp_total() { return warp_sum(s); }
 };
 template <>
 struct SqAcc<float> {
@@ -309,8 +315,9 @@ __device__ __forceinline__ SqAcc<R> qr_real_acc(const SqAcc<cplx<R>>& a) { retur
 
 // sqrt(a2), (|x| + sqrt(a2)) / sqrt(a2) and 1 / (|x| + sqrt(a2)) for the reflector, from the
 // hardware's float32 reciprocal (square root) and Newton / Halley steps: one
-// short dependent chain instead of a square root and two divisions, each right
-// to about an ulp.  float64: a2 in float32's range.
+// short dependent chain instead of a square root and two divisions.  Worst relative errors
+// measured against exact values over the range that comes here, in units of rounding
+// (2^-24, 2^-53): root 1.0, quotient 2.0, reciprocal 2.3.  float64: a2 in float32's range.
 __device__ __forceinline__ void qr_scalars(float a2, float ax, float& nrm, float& quo, float& inv) {
     float r = rsqrtf(a2);
     r = fmaf(0.5f * r, fmaf(-(a2 * r), r, 1.f), r);
